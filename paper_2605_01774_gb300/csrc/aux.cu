@@ -1,8 +1,7 @@
 // State transfer, read-outs, conservation reductions and the tensor pre-pass.
-#include <cfloat>
-
 #include "internal.h"
 #include "pull.cuh"
+#include "reduce.cuh"
 
 namespace elbm {
 
@@ -121,101 +120,6 @@ k_read(Field<Elem> f, Grid G, Tout* __restrict__ out, Tout* __restrict__ qout,
   }
 }
 
-// ----------------------------------------------------------------- reductions
-// Per block: sum phi, sum g ln(g/W) over g > 0, min g, count of non-finite g;
-// one partial per block, then a single block adds the partials in index order.
-template <typename Elem>
-__global__ void __launch_bounds__(256)
-k_reduce_partials(Field<Elem> f, Grid G, const float* __restrict__ src, double* __restrict__ part,
-                  const PopConsts<typename Storage<Elem>::real> k) {
-  using R = typename Storage<Elem>::real;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = blockIdx.z;
-  double m = 0.0, h = 0.0, gmin = DBL_MAX, bad = 0.0;
-  if (x < G.nx && y < G.ny) {
-    const int n = x + G.nx * (y + G.ny * z);
-    R g[Q];
-    pull_node<Elem, R>(g, f, G, x, y, z, k);
-    const double r = src != nullptr ? (double)k.src_half * (double)src[n] : 0.0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const double v = (double)g[i] + r * (double)k.E[i];
-      if (!isfinite(v)) {
-        bad += 1.0;
-        continue;
-      }
-      m += v;
-      if (v > 0.0) h += v * log(v / w_of(i));
-      gmin = fmin(gmin, v);
-    }
-  }
-  __shared__ double sm[4][8];
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  const int lane = tid & 31, wid = tid >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    m += __shfl_xor_sync(0xffffffffu, m, o);
-    h += __shfl_xor_sync(0xffffffffu, h, o);
-    gmin = fmin(gmin, __shfl_xor_sync(0xffffffffu, gmin, o));
-    bad += __shfl_xor_sync(0xffffffffu, bad, o);
-  }
-  if (lane == 0) {
-    sm[0][wid] = m;
-    sm[1][wid] = h;
-    sm[2][wid] = gmin;
-    sm[3][wid] = bad;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    const int nw = (blockDim.x * blockDim.y + 31) / 32;
-    double a = 0, b = 0, c = DBL_MAX, d = 0;
-    for (int w = 0; w < nw; ++w) {
-      a += sm[0][w];
-      b += sm[1][w];
-      c = fmin(c, sm[2][w]);
-      d += sm[3][w];
-    }
-    const size_t blk = blockIdx.x + (size_t)gridDim.x * (blockIdx.y + (size_t)gridDim.y * blockIdx.z);
-    part[4 * blk + 0] = a;
-    part[4 * blk + 1] = b;
-    part[4 * blk + 2] = c;
-    part[4 * blk + 3] = d;
-  }
-}
-
-__global__ void __launch_bounds__(1024) k_reduce_final(const double* __restrict__ part, size_t nblk,
-                                                       double* __restrict__ out4) {
-  __shared__ double sm[4][1024];
-  double a = 0, b = 0, c = DBL_MAX, d = 0;
-  for (size_t i = threadIdx.x; i < nblk; i += blockDim.x) {
-    a += part[4 * i];
-    b += part[4 * i + 1];
-    c = fmin(c, part[4 * i + 2]);
-    d += part[4 * i + 3];
-  }
-  sm[0][threadIdx.x] = a;
-  sm[1][threadIdx.x] = b;
-  sm[2][threadIdx.x] = c;
-  sm[3][threadIdx.x] = d;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      sm[0][threadIdx.x] += sm[0][threadIdx.x + s];
-      sm[1][threadIdx.x] += sm[1][threadIdx.x + s];
-      sm[2][threadIdx.x] = fmin(sm[2][threadIdx.x], sm[2][threadIdx.x + s]);
-      sm[3][threadIdx.x] += sm[3][threadIdx.x + s];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    out4[0] = sm[0][0];
-    out4[1] = sm[1][0];
-    out4[2] = sm[2][0];
-    out4[3] = sm[3][0];
-  }
-}
-
 // ---------------------------------------------------------------- tensor pre-pass
 // T = 2I - S = 12 D (I + 6 D)^-1 per node, in FP64 (Eq. method-s-from-d with
 // cs2 = 1/3, dt = 1), from Cartesian D or from (ln d_k, ZYZ angles).
@@ -331,12 +235,8 @@ cudaError_t read_t(const StateIO& S, void* out, void* q, int out_f32, int what, 
 template <typename Elem>
 cudaError_t reduce_t(const StateIO& S, double* scratch, double* out4, cudaStream_t s) {
   Grid G{S.nx, S.ny, S.nz, S.N, S.dirichlet};
-  dim3 b = block2d(S.nx), g = grid2d(b, S.nx, S.ny, S.nz);
-  k_reduce_partials<Elem><<<g, b, 0, s>>>(field_of<Elem>(S), G, S.src, scratch, consts_of<Elem>(S));
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_reduce_final<<<1, 1024, 0, s>>>(scratch, (size_t)g.x * g.y * g.z, out4);
-  return cudaGetLastError();
+  const auto& k = consts_of<Elem>(S);
+  return launch_reduce_t<Elem>(field_of<Elem>(S), G, S.src, (double)k.src_half, scratch, out4, k, s);
 }
 
 }  // namespace
@@ -361,10 +261,7 @@ cudaError_t launch_read_state(const StateIO& S, void* out, void* q, int out_f32,
   return cudaErrorInvalidValue;
 }
 
-size_t reduce_blocks(const StateIO& S) {
-  dim3 b = block2d(S.nx), g = grid2d(b, S.nx, S.ny, S.nz);
-  return (size_t)g.x * g.y * g.z;
-}
+size_t reduce_blocks(const StateIO& S) { return (size_t)reduce_grid(S.N); }
 
 cudaError_t launch_reduce(const StateIO& S, double* scratch, double* out4, cudaStream_t s) {
   switch (S.prec) {

@@ -22,6 +22,7 @@
 
 #include "../../include/elbm2d.h"
 #include "eqlog.cuh"
+#include "reduce.cuh"
 
 namespace {
 
@@ -242,70 +243,30 @@ __global__ void k_read2(const R* __restrict__ pops, Out* __restrict__ out, Grid2
   }
 }
 
-constexpr int RED_BLOCKS = 1024;
-
-// FP64 partial sums per block: mass, entropy over positive g, min g, non-finite count.
+// Partial sums per block: mass, entropy over positive g, min g, non-finite count.  A thread takes
+// three nodes at a time, 27 values that share one fixed-point scale (entropy.cuh).
 template <typename R>
 __global__ void __launch_bounds__(256) k_reduce2(const R* __restrict__ pops, size_t N, double* __restrict__ part) {
-  double m = 0.0, h = 0.0, gmin = 1.7976931348623157e308, bad = 0.0;
-  for (size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (size_t)gridDim.x * blockDim.x) {
-#pragma unroll
-    for (int i = 0; i < Q2; ++i) {
-      const double v = (double)pops[(size_t)i * N + n];
-      if (!isfinite(v)) {
-        bad += 1.0;
-        continue;
-      }
-      m += v;
-      if (v > 0.0) h += v * log(v / w2(i));
-      gmin = fmin(gmin, v);
-    }
-  }
-  __shared__ double sm[4][8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    m += __shfl_xor_sync(0xffffffffu, m, o);
-    h += __shfl_xor_sync(0xffffffffu, h, o);
-    gmin = fmin(gmin, __shfl_xor_sync(0xffffffffu, gmin, o));
-    bad += __shfl_xor_sync(0xffffffffu, bad, o);
-  }
-  if (lane == 0) {
-    sm[0][wid] = m;
-    sm[1][wid] = h;
-    sm[2][wid] = gmin;
-    sm[3][wid] = bad;
-  }
+  __shared__ long long table[elbm::LN_ENTRIES];
+  elbm::load_ln_table<2>(table);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0, b = 0, c = 1.7976931348623157e308, d = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      a += sm[0][w];
-      b += sm[1][w];
-      c = fmin(c, sm[2][w]);
-      d += sm[3][w];
-    }
-    part[4 * blockIdx.x + 0] = a;
-    part[4 * blockIdx.x + 1] = b;
-    part[4 * blockIdx.x + 2] = c;
-    part[4 * blockIdx.x + 3] = d;
+  double m = 0.0, h = 0.0, gmin = 1.7976931348623157e308;
+  unsigned bad = 0;
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (; n + 2 * stride < N; n += 3 * stride) {
+    R v[3 * Q2];
+#pragma unroll
+    for (int i = 0; i < 3 * Q2; ++i) v[i] = __ldg(pops + (size_t)(i % Q2) * N + n + (size_t)(i / Q2) * stride);
+    elbm::add_values<R, 3 * Q2>(v, [](int i) { return nnz2(i % Q2); }, table, m, h, gmin, bad);
   }
-}
-
-// Fixed-order sum of the partials (deterministic).
-__global__ void k_reduce2_final(const double* __restrict__ part, int nblk, double* __restrict__ out4) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double a = 0, b = 0, c = 1.7976931348623157e308, d = 0;
-  for (int i = 0; i < nblk; ++i) {
-    a += part[4 * i];
-    b += part[4 * i + 1];
-    c = fmin(c, part[4 * i + 2]);
-    d += part[4 * i + 3];
+  for (; n < N; n += stride) {
+    R v[Q2];
+#pragma unroll
+    for (int i = 0; i < Q2; ++i) v[i] = __ldg(pops + (size_t)i * N + n);
+    elbm::add_values<R, Q2>(v, [](int i) { return nnz2(i); }, table, m, h, gmin, bad);
   }
-  out4[0] = a;
-  out4[1] = b;
-  out4[2] = c;
-  out4[3] = d;
+  elbm::block_partials(m, h, gmin, (double)bad, part);
 }
 
 // T = 2I - S = 12 D (I + 6 D)^-1 per node from D3 [3][N] (FP32); counts non-SPD nodes.
@@ -572,7 +533,7 @@ elbm_status elbm2d_create(const int64_t dims[2], elbm_precision prec, void* cuda
   cudaError_t e = cudaSuccess;
   for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = cudaMalloc(&h->pops[b], Q2 * h->N * esize(h->prec));
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_counters, 2 * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_part, RED_BLOCKS * 4 * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_part, elbm::REDUCE_BLOCKS * 4 * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_out4, 4 * sizeof(double));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d_counters, 0, 2 * sizeof(unsigned long long), h->stream);
   if (e != cudaSuccess) {
@@ -706,11 +667,11 @@ elbm_status elbm2d_step(elbm2d_handle h, int64_t nsteps) {
 elbm_status elbm2d_reduce(elbm2d_handle h, double* mass, double* entropy, double* gmin, int64_t* n_fallback) {
   if (!h) return ELBM_ERR_ARG;
   if (!h->initialized) return fail(h, ELBM_ERR_STATE, "state not initialised");
-  const int nb = (int)std::min<size_t>((h->N + 255) / 256, RED_BLOCKS);
+  const int nb = elbm::reduce_grid(h->N);
   if (h->prec == 0) k_reduce2<double><<<nb, 256, 0, h->stream>>>((const double*)h->pops[h->cur], h->N, h->d_part);
   else k_reduce2<float><<<nb, 256, 0, h->stream>>>((const float*)h->pops[h->cur], h->N, h->d_part);
   CK2(cudaGetLastError(), "reduce");
-  k_reduce2_final<<<1, 32, 0, h->stream>>>(h->d_part, nb, h->d_out4);
+  elbm::k_reduce_final<<<1, 256, 0, h->stream>>>(h->d_part, nb, h->d_out4);
   CK2(cudaGetLastError(), "reduce final");
   double o[4];
   unsigned long long fb = 0;

@@ -1,6 +1,6 @@
 // Conservation diagnostics of a caller-held population state without any device
-// allocation: a grid-stride variant of the reduction in aux.cu whose partial sums
-// live in a file-scope device array instead of a buffer from cudaMalloc.
+// allocation: the reduction of reduce.cuh with its partial sums in a file-scope device
+// array instead of a buffer from cudaMalloc.
 //
 // Who needs it: code that must not allocate device memory at the moment it wants
 // the diagnostics -- a process whose device memory is already fully reserved by
@@ -12,13 +12,14 @@
 
 #include "../../include/elbm.h"
 #include "internal.h"
-#include "pull.cuh"
+#include "reduce.cuh"
 
 using namespace elbm;
 
 namespace {
 
-constexpr int kMaxPartials = 4096;  // blocks of the partial-sum kernel (grid-stride over nodes)
+constexpr int kMaxPartials = 4096;  // blocks of the partial-sum kernel that the array has room for
+static_assert(REDUCE_BLOCKS <= kMaxPartials, "partial sums fit the fixed array");
 constexpr int kMaxDevices = 64;
 
 // 4 doubles per block (mass, entropy, min g, non-finite count) + 4 for the final result:
@@ -31,95 +32,6 @@ std::mutex g_mu;
 // re-created (cudaDeviceReset), so the address is looked up again when the id changes.
 double* g_scratch_dev[kMaxDevices] = {};
 unsigned long long g_scratch_ctx[kMaxDevices] = {};
-
-template <typename Elem>
-__global__ void __launch_bounds__(256)
-k_partials_strided(Field<Elem> f, Grid G, const float* __restrict__ src, double* __restrict__ part,
-                   const PopConsts<typename Storage<Elem>::real> k) {
-  using R = typename Storage<Elem>::real;
-  double m = 0.0, h = 0.0, gmin = 1.7976931348623157e308, bad = 0.0;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x; n < G.N; n += stride) {
-    const int x = (int)(n % G.nx);
-    const int y = (int)((n / G.nx) % G.ny);
-    const int z = (int)(n / ((size_t)G.nx * G.ny));
-    R g[Q];
-    pull_node<Elem, R>(g, f, G, x, y, z, k);
-    const double r = src != nullptr ? 0.5 * (double)src[n] : 0.0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const double v = (double)g[i] + r * (double)k.E[i];
-      if (!isfinite(v)) {
-        bad += 1.0;
-        continue;
-      }
-      m += v;
-      if (v > 0.0) h += v * log(v / w_of(i));
-      gmin = fmin(gmin, v);
-    }
-  }
-  __shared__ double sm[4][8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    m += __shfl_xor_sync(0xffffffffu, m, o);
-    h += __shfl_xor_sync(0xffffffffu, h, o);
-    gmin = fmin(gmin, __shfl_xor_sync(0xffffffffu, gmin, o));
-    bad += __shfl_xor_sync(0xffffffffu, bad, o);
-  }
-  if (lane == 0) {
-    sm[0][wid] = m;
-    sm[1][wid] = h;
-    sm[2][wid] = gmin;
-    sm[3][wid] = bad;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0, b = 0, c = 1.7976931348623157e308, d = 0;
-    for (int w = 0; w < (int)(blockDim.x / 32); ++w) {
-      a += sm[0][w];
-      b += sm[1][w];
-      c = fmin(c, sm[2][w]);
-      d += sm[3][w];
-    }
-    part[4 * blockIdx.x + 0] = a;
-    part[4 * blockIdx.x + 1] = b;
-    part[4 * blockIdx.x + 2] = c;
-    part[4 * blockIdx.x + 3] = d;
-  }
-}
-
-__global__ void __launch_bounds__(256) k_final_strided(const double* __restrict__ part, int nblk,
-                                                       double* __restrict__ out4) {
-  __shared__ double sm[4][256];
-  double a = 0, b = 0, c = 1.7976931348623157e308, d = 0;
-  for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
-    a += part[4 * i];
-    b += part[4 * i + 1];
-    c = fmin(c, part[4 * i + 2]);
-    d += part[4 * i + 3];
-  }
-  sm[0][threadIdx.x] = a;
-  sm[1][threadIdx.x] = b;
-  sm[2][threadIdx.x] = c;
-  sm[3][threadIdx.x] = d;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      sm[0][threadIdx.x] += sm[0][threadIdx.x + s];
-      sm[1][threadIdx.x] += sm[1][threadIdx.x + s];
-      sm[2][threadIdx.x] = fmin(sm[2][threadIdx.x], sm[2][threadIdx.x + s]);
-      sm[3][threadIdx.x] += sm[3][threadIdx.x + s];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    out4[0] = sm[0][0];
-    out4[1] = sm[1][0];
-    out4[2] = sm[2][0];
-    out4[3] = sm[3][0];
-  }
-}
 
 // Unique id of the current context (driver entry points fetched through the runtime, so the
 // library needs no link against the driver library); 0 if it cannot be had.
@@ -186,14 +98,8 @@ template <typename Elem>
 cudaError_t launch(const void* pops, const float* scale, const Grid& G, const float* src, const double u[3],
                    const elbm_bc* bc, double* scratch, double* out4, cudaStream_t s) {
   using R = typename Storage<Elem>::real;
-  const size_t want = (G.N + 255) / 256;
-  const int nblk = (int)(want < (size_t)kMaxPartials ? want : (size_t)kMaxPartials);
   Field<Elem> f{static_cast<const Elem*>(pops), scale};
-  k_partials_strided<Elem><<<nblk, 256, 0, s>>>(f, G, src, scratch, pull_consts<R>(u, bc));
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_final_strided<<<1, 256, 0, s>>>(scratch, nblk, out4);
-  return cudaGetLastError();
+  return launch_reduce_t<Elem>(f, G, src, 0.5, scratch, out4, pull_consts<R>(u, bc), s);
 }
 
 bool device_ptr(const void* p) {
