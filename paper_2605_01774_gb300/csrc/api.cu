@@ -29,6 +29,7 @@ struct elbm_ctx {
   double u[3] = {0, 0, 0};
   elbm_params params{};
   PopConsts<double> kd{};
+  FixConsts fix{};                 // FP64: from kd
   PopConsts<float> kf{};
   unsigned long long* d_counters = nullptr;
   double* d_scratch = nullptr;
@@ -143,6 +144,7 @@ void rebuild_consts(elbm_ctx* h) {
   double T[6] = {0, 0, 0, 0, 0, 0};
   if (h->have_tensor && !h->tensor_field) complement6(h->D6, T);
   k.T = Sym6<double>{T[0], T[1], T[2], T[3], T[4], T[5]};
+  if (h->prec == 0) h->fix = fix_consts(k);
   PopConsts<float>& f = h->kf;
   for (int i = 0; i < Q; ++i) {
     f.E[i] = (float)k.E[i];
@@ -469,6 +471,7 @@ elbm_status elbm_step(elbm_handle h, int64_t nsteps) {
   L.counters = h->d_counters;
   L.kd = &h->kd;
   L.kf = &h->kf;
+  L.fix = &h->fix;
   L.variant = h->step_kernel;
   L.wait_limit = h->wait_limit;
   L.withheld = h->wait_withheld;

@@ -1,0 +1,85 @@
+// The collision of a pulled node with its source term, as every step kernel calls it: FP64 nodes of
+// a uniform velocity go through the fixed-point collision (fixed.cuh), all others through
+// collide_node.
+#pragma once
+#include "fixed.cuh"
+#include "pull.cuh"
+
+namespace elbm {
+
+// How a step kernel collides: in floating point with the closed-form stabilizer or with its exact
+// root, or (FP64) in fixed point.
+enum : int { CLOSED = 0, ROOT = 1, FIXED = 2 };
+
+// What a step kernel is given besides PopConsts: the fixed-point constants where it uses them.
+template <int MODE>
+struct StepConsts {};
+template <>
+struct StepConsts<FIXED> {
+  FixConsts fix;
+  PopConsts<double> pop;   // for step_node_f64, which takes its address
+};
+
+template <int MODE, typename Launch>
+inline StepConsts<MODE> step_consts(const Launch& L) {
+  StepConsts<MODE> c{};
+  if constexpr (MODE == FIXED) {
+    c.fix = *L.fix;
+    c.pop = *L.kd;
+  }
+  return c;
+}
+
+// Pull, FP64 collision and store of one of the few nodes that fixed point cannot hold: out of line,
+// so that it costs the others no registers.
+template <int VEL>
+__device__ __noinline__ bool step_node_f64(const Field<double>& in, const Grid& G, int n, const Sym6<double>& T, double r,
+                                           bool has_src, const PopConsts<double>& k, bool fallback, double* out) {
+  double g[Q], phi;
+  const int row = n / G.nx;
+  pull_node<double, double>(g, in, G, n - row * G.nx, row % G.ny, row / G.ny, k);
+  if (has_src) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] += r * k.E[i];
+  }
+  const bool took = collide_node<double, VEL>(g, T, k, fallback, phi);
+  Storage<double>::store(out, nullptr, (int)G.N, n, g, k.Ek, phi);
+  return took;
+}
+
+// Collides g_i + r E_i (has_src false: r is 0), g the populations pulled into node n of the lattice G
+// from `in`, with the node's T where has_T, else the uniform one, and stores the result in `pout`,
+// `sout`.  Returns whether the positivity fallback was taken; proj as Storage::store returns it.
+// keep: where fixed point keeps the node's integers.
+template <typename R, int VEL, int MODE, typename Elem, typename Keep>
+__device__ __forceinline__ bool collide_and_store(R (&g)[Q], const Field<Elem>& in, Elem* __restrict__ pout,
+                                                  float* __restrict__ sout, const Grid& G, int n, const Sym6<R>& T,
+                                                  bool has_T, R r, bool has_src, const PopConsts<R>& k,
+                                                  const StepConsts<MODE>& c, bool fallback, Keep& keep, bool& proj,
+                                                  const R* un = nullptr) {
+  if constexpr (MODE == FIXED) {
+    bool took;
+    const double t6[6] = {T.xx, T.xy, T.xz, T.yy, T.yz, T.zz};
+    proj = false;
+    if (collide_fixed<VEL>(g, has_T ? t6 : nullptr, r, has_src, fallback, c.fix, keep, took,
+                           [&](int i, double v) { pout[(size_t)i * G.N + n] = v; }))
+      return took;
+    return step_node_f64<VEL>(in, G, n, T, r, has_src, c.pop, fallback, pout);
+  } else {
+    if (has_src) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) g[i] += r * k.E[i];
+    }
+    R phi;
+    const bool took = collide_node<R, VEL, MODE == ROOT>(g, T, k, fallback, phi, un);
+    proj = Storage<Elem>::store(pout, sout, (int)G.N, n, g, k.Ek, phi, k.exact_mass != 0);
+    return took;
+  }
+}
+
+// Nothing to keep (floating-point collisions).
+struct KeepNone {};
+template <int MODE>
+using KeepLocal = typename std::conditional<MODE == FIXED, InLocal, KeepNone>::type;
+
+}  // namespace elbm

@@ -6,6 +6,7 @@
 #include <cstdint>
 
 #include "collide.cuh"
+#include "fixed.cuh"
 
 namespace elbm {
 
@@ -26,6 +27,7 @@ struct StepLaunch {
                                 // as their equilibrium shape, [4..5] row tickets
   const PopConsts<double>* kd;  // host copies, passed by value to the kernel
   const PopConsts<float>* kf;
+  const FixConsts* fix;         // FP64: of the fixed-point collision; fix->ok says whether it runs
   int variant;                  // 0 auto, 1 one thread per node with global gathers, 2 staged rows,
                                 // 3 staged rows with a producer warp and per-stage full/empty barriers
   long long wait_limit;         // staging waits of variants 2 and 3 give up after this many cycles

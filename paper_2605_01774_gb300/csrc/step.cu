@@ -1,6 +1,7 @@
 // Fused collide-stream kernel: one thread per node pulls its 27 populations,
 // collides them in registers (collide.cuh) and writes the 27 post-collision
 // values to its own node of the other buffer (coalesced writes, A/B buffers).
+#include "collide64.cuh"
 #include "internal.h"
 #include "pull.cuh"
 
@@ -11,44 +12,76 @@ namespace elbm {
 #define ELBM_STEP_MINB 3
 #endif
 template <typename Elem>
-constexpr int step_min_blocks() {
+__host__ __device__ constexpr int step_min_blocks() {
   return std::is_same<Elem, double>::value ? 1 : ELBM_STEP_MINB;
 }
 
-template <typename Elem, int VEL, bool ROOT>
-__global__ void __launch_bounds__(256, step_min_blocks<Elem>())
+// Threads per block and blocks per SM of the fixed-point FP64 kernel: 34 KB of shared memory per
+// 64 nodes (fixed.cuh) lets 6 blocks stand on an SM at 168 registers.  Measured on the 96 x 80 x 72
+// plume, 20 steps and their read-outs: 4 blocks 4.09, 6 blocks 3.69 ms; all loops unrolled, no
+// shared memory, 2 to 4 blocks of 128 3.97 to 4.24 ms (waiting for instructions); FP64 arithmetic
+// 10.7 ms.
+#ifndef ELBM_FIXED_THREADS
+#define ELBM_FIXED_THREADS 64
+#endif
+#ifndef ELBM_FIXED_MINB
+#define ELBM_FIXED_MINB 6
+#endif
+template <typename Elem, int MODE>
+__host__ __device__ constexpr int step_threads() {
+  return MODE == FIXED ? ELBM_FIXED_THREADS : 256;
+}
+template <typename Elem, int MODE>
+__host__ __device__ constexpr int step_blocks() {
+  return MODE == FIXED ? ELBM_FIXED_MINB : step_min_blocks<Elem>();
+}
+
+template <int MODE>
+using Kept = typename std::conditional<MODE == FIXED, InShared<ELBM_FIXED_THREADS>, KeepNone>::type;
+
+template <typename Elem, int VEL, int MODE>
+__global__ void __launch_bounds__(step_threads<Elem, MODE>(), step_blocks<Elem, MODE>())
 k_step(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G,
        const typename Storage<Elem>::real* __restrict__ T6,
        const float* __restrict__ src, const float* __restrict__ u3, int fallback,
-       unsigned long long* __restrict__ counters, const PopConsts<typename Storage<Elem>::real> k) {
+       unsigned long long* __restrict__ counters, const PopConsts<typename Storage<Elem>::real> k,
+       const __grid_constant__ StepConsts<MODE> c) {
   using R = typename Storage<Elem>::real;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = blockIdx.z;
+  int x, y, z;
+  if constexpr (MODE == FIXED) {
+    // long collisions: nodes in a row, so that no lane is lost to the ends of short rows
+    const unsigned m = blockIdx.x * (unsigned)step_threads<Elem, MODE>() + threadIdx.x, row = m / (unsigned)G.nx;
+    x = (int)(m - row * (unsigned)G.nx);
+    y = (int)(row % (unsigned)G.ny);
+    z = (int)(row / (unsigned)G.ny);
+  } else {
+    x = blockIdx.x * blockDim.x + threadIdx.x;
+    y = blockIdx.y * blockDim.y + threadIdx.y;
+    z = blockIdx.z;
+  }
+  __shared__ int64_t kept[MODE == FIXED ? KEPT * step_threads<Elem, MODE>() : 1];
   bool took = false, proj = false;
-  if (x < G.nx && y < G.ny) {
+  if (x < G.nx && y < G.ny && z < G.nz) {
     const int n = x + G.nx * (y + G.ny * z);
     R g[Q];
     pull_node<Elem, R>(g, in, G, x, y, z, k);
-    if (src != nullptr) {
-      // merged Strang half-steps of consecutive steps (Section 3.3)
-      const R r = k.src_step * R(__ldg(src + n));
-#pragma unroll
-      for (int i = 0; i < Q; ++i) g[i] += r * k.E[i];
-    }
+    // merged Strang half-steps of consecutive steps (Section 3.3)
+    const R r = src != nullptr ? k.src_step * R(__ldg(src + n)) : R(0);
     const Sym6<R> T = load_T<R>(T6, G.N, n, k.T);
-    R phi;
+    Kept<MODE> keep{};
+    if constexpr (MODE == FIXED) keep = Kept<MODE>{kept + threadIdx.x};
     if constexpr (VEL == 2) {
       const R un[3] = {R(__ldg(u3 + n)), R(__ldg(u3 + G.N + n)), R(__ldg(u3 + 2 * G.N + n))};
-      took = collide_node<R, 2, ROOT>(g, T, k, fallback != 0, phi, un);
+      took = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, c,
+                                             fallback != 0, keep, proj, un);
     } else {
-      took = collide_node<R, VEL, ROOT>(g, T, k, fallback != 0, phi);
+      took = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, c,
+                                             fallback != 0, keep, proj);
     }
-    proj = Storage<Elem>::store(pout, sout, G.N, n, g, k.Ek, phi, k.exact_mass != 0);
   }
   // one counter update per block
-  const int c = __syncthreads_count(took);
-  if (c != 0 && threadIdx.x == 0 && threadIdx.y == 0) atomicAdd(counters, (unsigned long long)c);
+  const int cnt = __syncthreads_count(took);
+  if (cnt != 0 && threadIdx.x == 0 && threadIdx.y == 0) atomicAdd(counters, (unsigned long long)cnt);
   if constexpr (Storage<Elem>::dev) {
     const int p = __syncthreads_count(proj);
     if (p != 0 && threadIdx.x == 0 && threadIdx.y == 0) atomicAdd(counters + 3, (unsigned long long)p);
@@ -60,17 +93,21 @@ static dim3 block_for(int nx) {
   return dim3(bx, 256 / bx, 1);
 }
 
-template <typename Elem, int VEL, bool ROOT>
+template <typename Elem, int VEL, int MODE>
 static cudaError_t launch_t(const StepLaunch& L, cudaStream_t s) {
   using R = typename Storage<Elem>::real;
   Field<Elem> in{static_cast<const Elem*>(L.pin), L.sin};
   Grid G{L.nx, L.ny, L.nz, L.N, L.dirichlet};
   dim3 b = block_for(L.nx);
   dim3 g((L.nx + b.x - 1) / b.x, (L.ny + b.y - 1) / b.y, L.nz);
+  if constexpr (MODE == FIXED) {
+    b = dim3(step_threads<Elem, MODE>());
+    g = dim3((unsigned)((L.N + b.x - 1) / b.x));
+  }
   const PopConsts<R>& k = *reinterpret_cast<const PopConsts<R>*>(std::is_same<R, double>::value ? (const void*)L.kd
                                                                                                : (const void*)L.kf);
-  k_step<Elem, VEL, ROOT><<<g, b, 0, s>>>(in, static_cast<Elem*>(L.pout), L.sout, G, static_cast<const R*>(L.T6), L.src,
-                                    L.u3, L.fallback, L.counters, k);
+  k_step<Elem, VEL, MODE><<<g, b, 0, s>>>(in, static_cast<Elem*>(L.pout), L.sout, G, static_cast<const R*>(L.T6), L.src,
+                                          L.u3, L.fallback, L.counters, k, step_consts<MODE>(L));
   return cudaGetLastError();
 }
 
@@ -78,9 +115,12 @@ template <typename Elem>
 static cudaError_t launch_v(const StepLaunch& L, cudaStream_t s) {
   // the exact root applies only where u != 0 (kappa = 0 at u = 0)
   const bool root = (std::is_same<Elem, double>::value ? L.kd->root : L.kf->root) != 0;
-  if (L.vel == 2) return root ? launch_t<Elem, 2, true>(L, s) : launch_t<Elem, 2, false>(L, s);
-  if (L.vel == 1) return root ? launch_t<Elem, 1, true>(L, s) : launch_t<Elem, 1, false>(L, s);
-  return launch_t<Elem, 0, false>(L, s);
+  if (L.vel == 2) return root ? launch_t<Elem, 2, ROOT>(L, s) : launch_t<Elem, 2, CLOSED>(L, s);
+  if (L.vel == 1 && root) return launch_t<Elem, 1, ROOT>(L, s);
+  if constexpr (std::is_same<Elem, double>::value) {
+    if (L.fix->ok) return L.vel == 1 ? launch_t<Elem, 1, FIXED>(L, s) : launch_t<Elem, 0, FIXED>(L, s);
+  }
+  return L.vel == 1 ? launch_t<Elem, 1, CLOSED>(L, s) : launch_t<Elem, 0, CLOSED>(L, s);
 }
 
 int step_variant(int prec, int nx, int vel, bool root, int requested) {

@@ -19,6 +19,7 @@
 #include <algorithm>
 
 #include "bulk.cuh"
+#include "collide64.cuh"
 #include "internal.h"
 #include "pull.cuh"
 
@@ -267,12 +268,14 @@ __device__ __forceinline__ int take_row(unsigned long long* counters, int nrows,
 // counters[0]: fallback nodes; [2]: set when a staging wait ran out; [3]: nodes stored as
 // their equilibrium shape (deviation storages, see Storage::store); [TICKET]: rows handed
 // out in this launch; [DONE]: blocks finished -- the last one resets both for the next launch.
-template <typename Elem, int VEL, bool ROOT, int WC>
+template <typename Elem, int VEL, int MODE, int WC>
 __global__ void __launch_bounds__(block_threads(WC), rows_min_blocks<Elem, WC>())
 k_step_rows(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G,
             const typename Storage<Elem>::real* __restrict__ T6, const float* __restrict__ src,
             const float* __restrict__ u3, int fallback, unsigned long long* __restrict__ counters,
-            long long wait_limit, int withheld, StageFmt sf, const PopConsts<typename Storage<Elem>::real> k) {
+            long long wait_limit, int withheld, StageFmt sf,
+            const PopConsts<typename Storage<Elem>::real> k,
+            const __grid_constant__ StepConsts<MODE> kc) {
   using R = typename Storage<Elem>::real;
   constexpr int BT = block_threads(WC), NW = BT / 32;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -372,22 +375,20 @@ k_step_rows(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
       }
       if (!valid) continue;
       if (G.dirichlet) abb_faces<Elem, R>(g, in, G, x, n, k);
-      if (src != nullptr) {
-        // merged Strang half-steps of consecutive steps (Section 3.3)
-        const R r = k.src_step * R(sv);
-#pragma unroll
-        for (int i = 0; i < Q; ++i) g[i] += r * k.E[i];
-      }
-      R phi;
-      bool t;
+      // merged Strang half-steps of consecutive steps (Section 3.3)
+      const R r = src != nullptr ? k.src_step * R(sv) : R(0);
+      KeepLocal<MODE> keep;
+      bool t, pr;
       if constexpr (VEL == 2) {
         const R un[3] = {R(__ldg(u3 + n)), R(__ldg(u3 + G.N + n)), R(__ldg(u3 + 2 * G.N + n))};
-        t = collide_node<R, 2, ROOT>(g, T, k, fallback != 0, phi, un);
+        t = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, kc,
+                                            fallback != 0, keep, pr, un);
       } else {
-        t = collide_node<R, VEL, ROOT>(g, T, k, fallback != 0, phi);
+        t = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, kc,
+                                            fallback != 0, keep, pr);
       }
       took += t ? 1u : 0u;
-      proj += Storage<Elem>::store(pout, sout, (int)G.N, n, g, k.Ek, phi, k.exact_mass != 0) ? 1u : 0u;
+      proj += pr ? 1u : 0u;
     }
   }
   if (stop) --it;                             // the aborted iteration
@@ -469,25 +470,26 @@ __host__ __device__ constexpr int pipe_blocks() {
   return std::is_same<Elem, double>::value ? 1 : ELBM_PIPE_BLOCKS;
 }
 
-template <typename Elem, int VEL, bool ROOT>
+template <typename Elem, int VEL, int MODE>
 __host__ __device__ constexpr int pipe_consumer_warps() {
   return std::is_same<Elem, double>::value ? 12
-                                            : ((VEL == 2 || ROOT) ? 7 : (Storage<Elem>::dev ? ELBM_PIPE_NC_DEV : ELBM_PIPE_NC));
+                                            : ((VEL == 2 || MODE == ROOT) ? 7 : (Storage<Elem>::dev ? ELBM_PIPE_NC_DEV : ELBM_PIPE_NC));
 }
 
-template <typename Elem, int VEL, bool ROOT>
+template <typename Elem, int VEL, int MODE>
 __host__ __device__ constexpr int pipe_threads() {
-  return 32 * (pipe_consumer_warps<Elem, VEL, ROOT>() + 1);
+  return 32 * (pipe_consumer_warps<Elem, VEL, MODE>() + 1);
 }
 
-template <typename Elem, int VEL, bool ROOT, int WC>
-__global__ void __launch_bounds__(pipe_threads<Elem, VEL, ROOT>(), pipe_blocks<Elem>())
+template <typename Elem, int VEL, int MODE, int WC>
+__global__ void __launch_bounds__(pipe_threads<Elem, VEL, MODE>(), pipe_blocks<Elem>())
 k_step_pipe(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G,
             const typename Storage<Elem>::real* __restrict__ T6, const float* __restrict__ src,
             const float* __restrict__ u3, int fallback, unsigned long long* __restrict__ counters,
-            long long wait_limit, int NS, const PopConsts<typename Storage<Elem>::real> k) {
+            long long wait_limit, int NS, const PopConsts<typename Storage<Elem>::real> k,
+            const __grid_constant__ StepConsts<MODE> kc) {
   using R = typename Storage<Elem>::real;
-  constexpr int NC = pipe_consumer_warps<Elem, VEL, ROOT>();
+  constexpr int NC = pipe_consumer_warps<Elem, VEL, MODE>();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t full[PIPE_MAX_STAGES], empty[PIPE_MAX_STAGES];
   __shared__ int s_row[PIPE_MAX_STAGES];
@@ -597,23 +599,21 @@ k_step_pipe(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
     if (x < W) {
       const int n = row * W + x;
       if (G.dirichlet) abb_faces<Elem, R>(g, in, G, x, n, k);
-      if (src != nullptr) {
-        // merged Strang half-steps of consecutive steps (Section 3.3)
-        const R r = k.src_step * R(__ldg(src + n));
-#pragma unroll
-        for (int i = 0; i < Q; ++i) g[i] += r * k.E[i];
-      }
+      // merged Strang half-steps of consecutive steps (Section 3.3)
+      const R r = src != nullptr ? k.src_step * R(__ldg(src + n)) : R(0);
       const Sym6<R> T = load_T<R>(T6, G.N, n, k.T);
-      R phi;
-      bool tk;
+      KeepLocal<MODE> keep;
+      bool tk, pr;
       if constexpr (VEL == 2) {
         const R un[3] = {R(__ldg(u3 + n)), R(__ldg(u3 + G.N + n)), R(__ldg(u3 + 2 * G.N + n))};
-        tk = collide_node<R, 2, ROOT>(g, T, k, fallback != 0, phi, un);
+        tk = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, kc,
+                                             fallback != 0, keep, pr, un);
       } else {
-        tk = collide_node<R, VEL, ROOT>(g, T, k, fallback != 0, phi);
+        tk = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, kc,
+                                             fallback != 0, keep, pr);
       }
       took += tk ? 1u : 0u;
-      proj += Storage<Elem>::store(pout, sout, (int)G.N, n, g, k.Ek, phi, k.exact_mass != 0) ? 1u : 0u;
+      proj += pr ? 1u : 0u;
     }
   }
 #pragma unroll
@@ -628,9 +628,9 @@ k_step_pipe(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
 
 namespace {
 
-// Blocks of k_step_rows<Elem, VEL, ROOT, WC> resident per SM with `dyn` bytes of stages (0: not
+// Blocks of k_step_rows<Elem, VEL, MODE, WC> resident per SM with `dyn` bytes of stages (0: not
 // launchable); raises the kernel's dynamic shared-memory limit as needed.  Cached per (device, dyn).
-template <typename Elem, int VEL, bool ROOT, int WC>
+template <typename Elem, int VEL, int MODE, int WC>
 int rows_occupancy(size_t dyn) {
   static int c_dev[4] = {-1, -1, -1, -1}, c_nb[4] = {0, 0, 0, 0};
   static size_t c_dyn[4] = {0, 0, 0, 0};
@@ -642,11 +642,11 @@ int rows_occupancy(size_t dyn) {
   int nb = 0;
   // raise (never lower) the kernel's limit: another layout may already have been launched
   cudaFuncAttributes fa;
-  const int cur = cudaFuncGetAttributes(&fa, k_step_rows<Elem, VEL, ROOT, WC>) == cudaSuccess
+  const int cur = cudaFuncGetAttributes(&fa, k_step_rows<Elem, VEL, MODE, WC>) == cudaSuccess
                       ? fa.maxDynamicSharedSizeBytes : 0;
-  if ((cur >= (int)dyn || cudaFuncSetAttribute(k_step_rows<Elem, VEL, ROOT, WC>,
+  if ((cur >= (int)dyn || cudaFuncSetAttribute(k_step_rows<Elem, VEL, MODE, WC>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) == cudaSuccess) &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step_rows<Elem, VEL, ROOT, WC>, block_threads(WC), dyn) ==
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step_rows<Elem, VEL, MODE, WC>, block_threads(WC), dyn) ==
           cudaSuccess) {
     c_dev[next] = dev;
     c_dyn[next] = dyn;
@@ -658,15 +658,15 @@ int rows_occupancy(size_t dyn) {
   return 0;
 }
 
-template <typename Elem, int VEL, bool ROOT, int WC>
+template <typename Elem, int VEL, int MODE, int WC>
 cudaError_t launch_rows_t(const StepLaunch& L, cudaStream_t s) {
   using R = typename Storage<Elem>::real;
   // stage the T-field and source rows too where that keeps the resident blocks per SM
   const StageFmt base = stage_fmt<Elem>(L.nx, false, false, 0);
   StageFmt sf = stage_fmt<Elem>(L.nx, L.T6 != nullptr, L.src != nullptr, ELBM_ROWS_FIELD_BUDGET);
-  int nb = rows_occupancy<Elem, VEL, ROOT, WC>(STAGES * (size_t)base.bytes);
+  int nb = rows_occupancy<Elem, VEL, MODE, WC>(STAGES * (size_t)base.bytes);
   if (sf.bytes != base.bytes) {
-    const int nbf = rows_occupancy<Elem, VEL, ROOT, WC>(STAGES * (size_t)sf.bytes);
+    const int nbf = rows_occupancy<Elem, VEL, MODE, WC>(STAGES * (size_t)sf.bytes);
     if (nbf >= nb && nbf > 0) nb = nbf;
     else sf = base;
   }
@@ -679,7 +679,7 @@ cudaError_t launch_rows_t(const StepLaunch& L, cudaStream_t s) {
   static size_t c_max = 0;
   const size_t dyn = STAGES * (size_t)sf.bytes;
   if (dev != c_dev || dyn > c_max) {
-    if (cudaFuncSetAttribute(k_step_rows<Elem, VEL, ROOT, WC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(k_step_rows<Elem, VEL, MODE, WC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)std::max(dyn, dev == c_dev ? c_max : (size_t)0)) != cudaSuccess)
       return cudaGetLastError();
     c_max = std::max(dyn, dev == c_dev ? c_max : (size_t)0);
@@ -692,22 +692,26 @@ cudaError_t launch_rows_t(const StepLaunch& L, cudaStream_t s) {
   Grid G{L.nx, L.ny, L.nz, L.N, L.dirichlet};
   const PopConsts<R>& k = *reinterpret_cast<const PopConsts<R>*>(std::is_same<R, double>::value ? (const void*)L.kd
                                                                                                : (const void*)L.kf);
-  k_step_rows<Elem, VEL, ROOT, WC><<<grid, block_threads(WC), STAGES * (size_t)sf.bytes, s>>>(
+  k_step_rows<Elem, VEL, MODE, WC><<<grid, block_threads(WC), STAGES * (size_t)sf.bytes, s>>>(
       in, static_cast<Elem*>(L.pout), L.sout, G, static_cast<const R*>(L.T6), L.src, L.u3, L.fallback, L.counters,
-      L.wait_limit > 0 ? L.wait_limit : WAIT_LIMIT, L.withheld, sf, k);
+      L.wait_limit > 0 ? L.wait_limit : WAIT_LIMIT, L.withheld, sf, k, step_consts<MODE>(L));
   return cudaGetLastError();
 }
 
 template <typename Elem>
 cudaError_t launch_rows_v(const StepLaunch& L, cudaStream_t s) {
   const bool root = (std::is_same<Elem, double>::value ? L.kd->root : L.kf->root) != 0;
-  if (L.vel == 2) return root ? launch_rows_t<Elem, 2, true, 0>(L, s) : launch_rows_t<Elem, 2, false, 0>(L, s);
-  if (root) return L.vel == 1 ? launch_rows_t<Elem, 1, true, 0>(L, s) : launch_rows_t<Elem, 0, false, 0>(L, s);
-  // closed-form stabilizer, uniform velocity: row lengths 256, 384 and 512 compiled in
-  if (L.nx == 256) return L.vel == 1 ? launch_rows_t<Elem, 1, false, 256>(L, s) : launch_rows_t<Elem, 0, false, 256>(L, s);
-  if (L.nx == 512) return L.vel == 1 ? launch_rows_t<Elem, 1, false, 512>(L, s) : launch_rows_t<Elem, 0, false, 512>(L, s);
-  if (L.nx == 384) return L.vel == 1 ? launch_rows_t<Elem, 1, false, 384>(L, s) : launch_rows_t<Elem, 0, false, 384>(L, s);
-  return L.vel == 1 ? launch_rows_t<Elem, 1, false, 0>(L, s) : launch_rows_t<Elem, 0, false, 0>(L, s);
+  if (L.vel == 2) return root ? launch_rows_t<Elem, 2, ROOT, 0>(L, s) : launch_rows_t<Elem, 2, CLOSED, 0>(L, s);
+  if (root && L.vel == 1) return launch_rows_t<Elem, 1, ROOT, 0>(L, s);
+  if constexpr (std::is_same<Elem, double>::value) {
+    if (L.fix->ok) return L.vel == 1 ? launch_rows_t<Elem, 1, FIXED, 0>(L, s) : launch_rows_t<Elem, 0, FIXED, 0>(L, s);
+  } else if (!root) {
+    // closed-form stabilizer, uniform velocity: row lengths 256, 384 and 512 compiled in
+    if (L.nx == 256) return L.vel == 1 ? launch_rows_t<Elem, 1, CLOSED, 256>(L, s) : launch_rows_t<Elem, 0, CLOSED, 256>(L, s);
+    if (L.nx == 512) return L.vel == 1 ? launch_rows_t<Elem, 1, CLOSED, 512>(L, s) : launch_rows_t<Elem, 0, CLOSED, 512>(L, s);
+    if (L.nx == 384) return L.vel == 1 ? launch_rows_t<Elem, 1, CLOSED, 384>(L, s) : launch_rows_t<Elem, 0, CLOSED, 384>(L, s);
+  }
+  return L.vel == 1 ? launch_rows_t<Elem, 1, CLOSED, 0>(L, s) : launch_rows_t<Elem, 0, CLOSED, 0>(L, s);
 }
 
 }  // namespace
@@ -729,10 +733,10 @@ int pipe_stages_for(int prec, int W, int nc) {
   return ns;
 }
 
-template <typename Elem, int VEL, bool ROOT, int WC>
+template <typename Elem, int VEL, int MODE, int WC>
 cudaError_t launch_pipe_t(const StepLaunch& L, cudaStream_t s) {
   using R = typename Storage<Elem>::real;
-  constexpr int NC = pipe_consumer_warps<Elem, VEL, ROOT>();
+  constexpr int NC = pipe_consumer_warps<Elem, VEL, MODE>();
   const int ns = pipe_stages_for(L.prec, L.nx, NC);
   if (ns == 0) return cudaErrorNotSupported;
   const size_t dyn = (size_t)ns * stage_bytes<Elem>(L.nx);
@@ -741,7 +745,7 @@ cudaError_t launch_pipe_t(const StepLaunch& L, cudaStream_t s) {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   if (dev != c_dev || dyn > c_dyn) {
-    cudaError_t e = cudaFuncSetAttribute(k_step_pipe<Elem, VEL, ROOT, WC>,
+    cudaError_t e = cudaFuncSetAttribute(k_step_pipe<Elem, VEL, MODE, WC>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e != cudaSuccess) return e;
     c_dev = dev;
@@ -754,22 +758,26 @@ cudaError_t launch_pipe_t(const StepLaunch& L, cudaStream_t s) {
   Grid G{L.nx, L.ny, L.nz, L.N, L.dirichlet};
   const PopConsts<R>& k = *reinterpret_cast<const PopConsts<R>*>(std::is_same<R, double>::value ? (const void*)L.kd
                                                                                                : (const void*)L.kf);
-  k_step_pipe<Elem, VEL, ROOT, WC><<<grid, pipe_threads<Elem, VEL, ROOT>(), dyn, s>>>(
+  k_step_pipe<Elem, VEL, MODE, WC><<<grid, pipe_threads<Elem, VEL, MODE>(), dyn, s>>>(
       in, static_cast<Elem*>(L.pout), L.sout, G, static_cast<const R*>(L.T6), L.src, L.u3, L.fallback, L.counters,
-      L.wait_limit > 0 ? L.wait_limit : WAIT_LIMIT, ns, k);
+      L.wait_limit > 0 ? L.wait_limit : WAIT_LIMIT, ns, k, step_consts<MODE>(L));
   return cudaGetLastError();
 }
 
 template <typename Elem>
 cudaError_t launch_pipe_v(const StepLaunch& L, cudaStream_t s) {
   const bool root = (std::is_same<Elem, double>::value ? L.kd->root : L.kf->root) != 0;
-  if (L.vel == 2) return root ? launch_pipe_t<Elem, 2, true, 0>(L, s) : launch_pipe_t<Elem, 2, false, 0>(L, s);
-  if (root) return L.vel == 1 ? launch_pipe_t<Elem, 1, true, 0>(L, s) : launch_pipe_t<Elem, 0, false, 0>(L, s);
-  // closed-form stabilizer, uniform velocity: row lengths 256, 384 and 512 compiled in
-  if (L.nx == 256) return L.vel == 1 ? launch_pipe_t<Elem, 1, false, 256>(L, s) : launch_pipe_t<Elem, 0, false, 256>(L, s);
-  if (L.nx == 512) return L.vel == 1 ? launch_pipe_t<Elem, 1, false, 512>(L, s) : launch_pipe_t<Elem, 0, false, 512>(L, s);
-  if (L.nx == 384) return L.vel == 1 ? launch_pipe_t<Elem, 1, false, 384>(L, s) : launch_pipe_t<Elem, 0, false, 384>(L, s);
-  return L.vel == 1 ? launch_pipe_t<Elem, 1, false, 0>(L, s) : launch_pipe_t<Elem, 0, false, 0>(L, s);
+  if (L.vel == 2) return root ? launch_pipe_t<Elem, 2, ROOT, 0>(L, s) : launch_pipe_t<Elem, 2, CLOSED, 0>(L, s);
+  if (root && L.vel == 1) return launch_pipe_t<Elem, 1, ROOT, 0>(L, s);
+  if constexpr (std::is_same<Elem, double>::value) {
+    if (L.fix->ok) return L.vel == 1 ? launch_pipe_t<Elem, 1, FIXED, 0>(L, s) : launch_pipe_t<Elem, 0, FIXED, 0>(L, s);
+  } else if (!root) {
+    // closed-form stabilizer, uniform velocity: row lengths 256, 384 and 512 compiled in
+    if (L.nx == 256) return L.vel == 1 ? launch_pipe_t<Elem, 1, CLOSED, 256>(L, s) : launch_pipe_t<Elem, 0, CLOSED, 256>(L, s);
+    if (L.nx == 512) return L.vel == 1 ? launch_pipe_t<Elem, 1, CLOSED, 512>(L, s) : launch_pipe_t<Elem, 0, CLOSED, 512>(L, s);
+    if (L.nx == 384) return L.vel == 1 ? launch_pipe_t<Elem, 1, CLOSED, 384>(L, s) : launch_pipe_t<Elem, 0, CLOSED, 384>(L, s);
+  }
+  return L.vel == 1 ? launch_pipe_t<Elem, 1, CLOSED, 0>(L, s) : launch_pipe_t<Elem, 0, CLOSED, 0>(L, s);
 }
 
 }  // namespace
