@@ -22,6 +22,7 @@
 
 #include "../../include/elbm2d.h"
 #include "eqlog.cuh"
+#include "launch.cuh"
 #include "reduce.cuh"
 
 namespace {
@@ -150,8 +151,9 @@ struct Grid2 {
 // Rows y handled by this thread: y0, y0 + ystride, ...
 template <typename R, int VEL>
 __global__ void __launch_bounds__(256)
-k_step2(const R* __restrict__ in, R* __restrict__ out, Grid2 G, const R* __restrict__ T3,
+k_step2(const R* in, R* out, Grid2 G, const R* __restrict__ T3,
         const float* __restrict__ u2, int fallback, unsigned long long* __restrict__ counters, const Consts2<R> k) {
+  elbm::wait_for_previous();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int ystride = gridDim.y * blockDim.y;
   unsigned took = 0;
@@ -163,7 +165,7 @@ k_step2(const R* __restrict__ in, R* __restrict__ out, Grid2 G, const R* __restr
     const int ys[3] = {(y + 1 == G.ny ? 0 : y + 1) * G.nx, y * G.nx, (y == 0 ? G.ny - 1 : y - 1) * G.nx};
     R g[Q2];
 #pragma unroll
-    for (int i = 0; i < Q2; ++i) g[i] = __ldg(in + (size_t)i * G.N + (size_t)(xs[cx2(i) + 1] + ys[cy2(i) + 1]));
+    for (int i = 0; i < Q2; ++i) g[i] = in[(size_t)i * G.N + (size_t)(xs[cx2(i) + 1] + ys[cy2(i) + 1])];
     R txx = k.txx, txy = k.txy, tyy = k.tyy;
     if (T3 != nullptr) {
       txx = __ldg(T3 + n);
@@ -433,10 +435,8 @@ cudaError_t launch_step2(elbm2d_ctx* h) {
   R* out = static_cast<R*>(h->pops[1 - h->cur]);
   const R* T3 = h->tensor_field ? static_cast<const R*>(h->T3) : nullptr;
   const int fb = h->params.fallback;
-  if (vel == 2) k_step2<R, 2><<<grid, block, 0, h->stream>>>(in, out, G, T3, h->u2, fb, h->d_counters, k);
-  else if (vel == 1) k_step2<R, 1><<<grid, block, 0, h->stream>>>(in, out, G, T3, nullptr, fb, h->d_counters, k);
-  else k_step2<R, 0><<<grid, block, 0, h->stream>>>(in, out, G, T3, nullptr, fb, h->d_counters, k);
-  return cudaGetLastError();
+  auto kernel = vel == 2 ? k_step2<R, 2> : (vel == 1 ? k_step2<R, 1> : k_step2<R, 0>);
+  return elbm::launch_next(kernel, grid, block, 0, h->stream, in, out, G, T3, h->u2, fb, h->d_counters, k);
 }
 
 elbm_status write_state(elbm2d_ctx* h, const void* in, elbm_dtype dt, int from_phi) {

@@ -1,0 +1,42 @@
+// Launches of kernels that follow one another on a stream, each reading what the one before wrote.
+//
+// A launch that waits for the previous kernel to end before it is set up costs about 2 us per step;
+// with programmatic stream serialisation the next kernel's blocks are placed while the last ones of
+// this kernel finish and wait inside, in wait_for_previous(), for its memory.  Measured: an empty
+// kernel 2.05 -> 1.5 us; a step with 121 x 75 x 50 nodes (FP32, tensor field) 22.7 -> 19.5 us, 32^3
+// (FP64) 8.3 -> 7.2 us, 24^3 (FP32) 4.2 -> 3.8 us.
+//
+// What a step reads after the wait it reads with plain loads: its L1 lines date from its own launch
+// or later, and between that and the wait only the previous step runs, which loads the other buffer.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <utility>
+
+namespace elbm {
+
+// First statement of every kernel launched by launch_next: lets the next launch be placed, then
+// waits until the kernel before this one has ended and its writes are visible.  Nothing that an
+// earlier kernel writes may be touched before it.
+__device__ __forceinline__ void wait_for_previous() {
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
+}
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_next(void (*kernel)(Params...), dim3 grid, dim3 block, size_t shared, cudaStream_t s,
+                               Args&&... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = shared;
+  c.stream = s;
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &a;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, std::forward<Args>(args)...);
+}
+
+}  // namespace elbm

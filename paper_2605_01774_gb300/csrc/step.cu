@@ -3,6 +3,7 @@
 // values to its own node of the other buffer (coalesced writes, A/B buffers).
 #include "collide64.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "pull.cuh"
 
 namespace elbm {
@@ -47,6 +48,7 @@ k_step(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G
        unsigned long long* __restrict__ counters, const PopConsts<typename Storage<Elem>::real> k,
        const __grid_constant__ StepConsts<MODE> c) {
   using R = typename Storage<Elem>::real;
+  wait_for_previous();
   int x, y, z;
   if constexpr (MODE == FIXED) {
     // long collisions: nodes in a row, so that no lane is lost to the ends of short rows
@@ -106,9 +108,8 @@ static cudaError_t launch_t(const StepLaunch& L, cudaStream_t s) {
   }
   const PopConsts<R>& k = *reinterpret_cast<const PopConsts<R>*>(std::is_same<R, double>::value ? (const void*)L.kd
                                                                                                : (const void*)L.kf);
-  k_step<Elem, VEL, MODE><<<g, b, 0, s>>>(in, static_cast<Elem*>(L.pout), L.sout, G, static_cast<const R*>(L.T6), L.src,
-                                          L.u3, L.fallback, L.counters, k, step_consts<MODE>(L));
-  return cudaGetLastError();
+  return launch_next(k_step<Elem, VEL, MODE>, g, b, 0, s, in, static_cast<Elem*>(L.pout), L.sout, G,
+                     static_cast<const R*>(L.T6), L.src, L.u3, L.fallback, L.counters, k, step_consts<MODE>(L));
 }
 
 template <typename Elem>

@@ -21,6 +21,7 @@
 #include "bulk.cuh"
 #include "collide64.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "pull.cuh"
 
 #ifndef ELBM_ROWS_STAGES
@@ -298,6 +299,7 @@ k_step_rows(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
     mbar_fence_init();
   }
   __syncthreads();
+  wait_for_previous();
   // thread 0: the ticket of the next row to issue, taken one row ahead so that the atomic's
   // round trip overlaps a row of collisions
   unsigned long long pend = 0;
@@ -512,6 +514,7 @@ k_step_pipe(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
     abort_flag = 0;
   }
   __syncthreads();
+  wait_for_previous();
   volatile int* vabort = &abort_flag;
 
   if (warp == NC) {
@@ -692,10 +695,10 @@ cudaError_t launch_rows_t(const StepLaunch& L, cudaStream_t s) {
   Grid G{L.nx, L.ny, L.nz, L.N, L.dirichlet};
   const PopConsts<R>& k = *reinterpret_cast<const PopConsts<R>*>(std::is_same<R, double>::value ? (const void*)L.kd
                                                                                                : (const void*)L.kf);
-  k_step_rows<Elem, VEL, MODE, WC><<<grid, block_threads(WC), STAGES * (size_t)sf.bytes, s>>>(
-      in, static_cast<Elem*>(L.pout), L.sout, G, static_cast<const R*>(L.T6), L.src, L.u3, L.fallback, L.counters,
+  return launch_next(
+      k_step_rows<Elem, VEL, MODE, WC>, dim3(grid), dim3(block_threads(WC)), STAGES * (size_t)sf.bytes, s, in,
+      static_cast<Elem*>(L.pout), L.sout, G, static_cast<const R*>(L.T6), L.src, L.u3, L.fallback, L.counters,
       L.wait_limit > 0 ? L.wait_limit : WAIT_LIMIT, L.withheld, sf, k, step_consts<MODE>(L));
-  return cudaGetLastError();
 }
 
 template <typename Elem>
@@ -758,10 +761,10 @@ cudaError_t launch_pipe_t(const StepLaunch& L, cudaStream_t s) {
   Grid G{L.nx, L.ny, L.nz, L.N, L.dirichlet};
   const PopConsts<R>& k = *reinterpret_cast<const PopConsts<R>*>(std::is_same<R, double>::value ? (const void*)L.kd
                                                                                                : (const void*)L.kf);
-  k_step_pipe<Elem, VEL, MODE, WC><<<grid, pipe_threads<Elem, VEL, MODE>(), dyn, s>>>(
-      in, static_cast<Elem*>(L.pout), L.sout, G, static_cast<const R*>(L.T6), L.src, L.u3, L.fallback, L.counters,
+  return launch_next(
+      k_step_pipe<Elem, VEL, MODE, WC>, dim3(grid), dim3(pipe_threads<Elem, VEL, MODE>()), dyn, s, in,
+      static_cast<Elem*>(L.pout), L.sout, G, static_cast<const R*>(L.T6), L.src, L.u3, L.fallback, L.counters,
       L.wait_limit > 0 ? L.wait_limit : WAIT_LIMIT, ns, k, step_consts<MODE>(L));
-  return cudaGetLastError();
 }
 
 template <typename Elem>

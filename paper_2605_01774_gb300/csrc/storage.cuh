@@ -61,12 +61,13 @@ struct Storage {
   static constexpr bool dev = !(std::is_same<Elem, double>::value || std::is_same<Elem, float>::value);
   using real = typename std::conditional<std::is_same<Elem, double>::value, double, float>::type;
 
-  // Value of population i stored at node `src` (i is a constant after unrolling).
-  static __device__ __forceinline__ real load(const Elem* __restrict__ pops, const float* __restrict__ scale,
-                                              int N, int i, int src, real E_i) {
-    const Elem v = __ldg(pops + (i * N + src));  // 27 N < 2^31 is checked at creation
+  // Value of population i stored at node `src` (i is a constant after unrolling).  Plain loads, not
+  // read-only ones: a step kernel may be resident while the kernel before it still writes this
+  // buffer (launch.cuh), and read-only loads may be moved across that wait.
+  static __device__ __forceinline__ real load(const Elem* pops, const float* scale, int N, int i, int src, real E_i) {
+    const Elem v = pops[i * N + src];            // 27 N < 2^31 is checked at creation
     if constexpr (dev) {
-      const float s = __ldg(scale + src);
+      const float s = scale[src];
       return s * Codec<Elem>::fma_pow2(v, qexp_of(i), E_i);
     } else {
       return v;
