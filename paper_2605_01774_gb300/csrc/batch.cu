@@ -167,13 +167,11 @@ __global__ void k_batch_write(const DomainInfo* dom, const int* tile_dom, const 
   }
 }
 
-__global__ void k_batch_read(const DomainInfo* dom, const int* tile_dom, const int* tile_first, int ntiles,
-                             const float* __restrict__ buf, float* __restrict__ phi, float* __restrict__ pops,
-                             int only_dom) {
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int di = tile_dom[t];
-    if (only_dom >= 0 && di != only_dom) continue;
-    const DomainInfo d = dom[di];
+// Tiles [t0, t1): phi of their nodes in the concatenated order, or (one domain's tiles) its populations.
+__global__ void k_batch_read(const DomainInfo* dom, const int* tile_dom, const int* tile_first, int t0, int t1,
+                             const float* __restrict__ buf, float* __restrict__ phi, float* __restrict__ pops) {
+  for (int t = t0 + blockIdx.x; t < t1; t += gridDim.x) {
+    const DomainInfo d = dom[tile_dom[t]];
     const int local = tile_first[t] + threadIdx.x;
     const int n = d.n, N = n * n * n;
     if (local >= N) continue;
@@ -221,6 +219,7 @@ struct elbm_batch_ctx {
   cudaStream_t own_stream = nullptr;   // created when the caller passed the default stream
   int in_graph = -1;
   int tile = 256, blocks_per_sm = 0, nsm = 0;
+  int step_blocks = 0;         // mode 1: blocks per SM of one wave
   int ntiles = 0;
   DomainInfo* d_dom = nullptr;
   int* d_tile_dom = nullptr;
@@ -403,7 +402,11 @@ elbm_status elbm_batch_create(int32_t ndom, const int32_t* edges, const double* 
   }
   int bps = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_batch_persistent, 256, 0);
-  h->blocks_per_sm = std::max(1, bps);
+  // Two blocks per SM until the autotuner is asked: a third one only has more rows of more planes
+  // open at once, and DRAM serves them more slowly (512 domains of 16^3 to 96^3, 10 steps: 61.7 ms
+  // with three, 52.6 with two; with two at 128 registers 52.5).
+  h->blocks_per_sm = std::max(1, std::min(2, bps));
+  h->step_blocks = std::max(1, bps);   // separate launches: 57.4 ms with three, 59.0 with two
   if (rebuild_tiles(h) != ELBM_OK) {
     elbm_batch_destroy(h);
     return ELBM_ERR_CUDA;
@@ -526,7 +529,7 @@ elbm_status elbm_batch_step(elbm_batch_handle h, int64_t nsteps, int32_t mode) {
   } else {
     BatchArgs a = args_of(h);
     int parity = h->parity;
-    const int grid = h->blocks_per_sm * h->nsm * 4;
+    const int grid = h->step_blocks * h->nsm * 4;
     for (int64_t s = 0; s < nsteps && e == cudaSuccess; ++s) {
       k_batch_step<<<grid, h->tile, 0, h->stream>>>(a, parity);
       e = cudaGetLastError();
@@ -609,7 +612,7 @@ elbm_status elbm_batch_autotune(elbm_batch_handle h, int32_t steps_per_trial, in
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  h->blocks_per_sm = best_b;
+  h->blocks_per_sm = h->step_blocks = best_b;
   if (h->tile != best_t) {
     h->tile = best_t;
     elbm_status s = rebuild_tiles(h);
@@ -627,8 +630,8 @@ elbm_status elbm_batch_read_phi(elbm_batch_handle h, float* phi) {
   float* dst = phi;
   if (host) BCK(cudaMallocAsync((void**)&dst, h->total * sizeof(float), h->stream), "cudaMallocAsync");
   const int grid = std::min(h->ntiles, 65535 * 8);
-  k_batch_read<<<grid, h->tile, 0, h->stream>>>(h->d_dom, h->d_tile_dom, h->d_tile_first, h->ntiles,
-                                               h->buf[h->parity], dst, nullptr, -1);
+  k_batch_read<<<grid, h->tile, 0, h->stream>>>(h->d_dom, h->d_tile_dom, h->d_tile_first, 0, h->ntiles,
+                                               h->buf[h->parity], dst, nullptr);
   BCK(cudaGetLastError(), "read kernel");
   if (host) {
     BCK(cudaMemcpyAsync(phi, dst, h->total * sizeof(float), cudaMemcpyDeviceToHost, h->stream), "memcpy");
@@ -645,9 +648,13 @@ elbm_status elbm_batch_read_populations(elbm_batch_handle h, int32_t domain, flo
   const bool host = !dptr(out);
   float* dst = out;
   if (host) BCK(cudaMallocAsync((void**)&dst, 27 * N * sizeof(float), h->stream), "cudaMallocAsync");
-  const int grid = std::min(h->ntiles, 65535 * 8);
-  k_batch_read<<<grid, h->tile, 0, h->stream>>>(h->d_dom, h->d_tile_dom, h->d_tile_first, h->ntiles,
-                                               h->buf[h->parity], nullptr, dst, domain);
+  // the domain's tiles alone
+  const auto tiles_of = [&](int d) { return (int)(((long long)h->edges[d] * h->edges[d] * h->edges[d] + h->tile - 1) / h->tile); };
+  int t0 = 0;
+  for (int d = 0; d < domain; ++d) t0 += tiles_of(d);
+  const int grid = std::min(tiles_of(domain), 65535 * 8);
+  k_batch_read<<<grid, h->tile, 0, h->stream>>>(h->d_dom, h->d_tile_dom, h->d_tile_first, t0, t0 + tiles_of(domain),
+                                               h->buf[h->parity], nullptr, dst);
   BCK(cudaGetLastError(), "read kernel");
   if (host) {
     BCK(cudaMemcpyAsync(out, dst, 27 * N * sizeof(float), cudaMemcpyDeviceToHost, h->stream), "memcpy");
