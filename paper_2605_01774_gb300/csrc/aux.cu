@@ -1,5 +1,6 @@
 // State transfer, read-outs, conservation reductions and the tensor pre-pass.
 #include "internal.h"
+#include "launch.cuh"
 #include "pull.cuh"
 #include "reduce.cuh"
 
@@ -7,15 +8,17 @@ namespace elbm {
 
 namespace {
 
-dim3 block2d(int nx) {
-  int bx = nx >= 256 ? 256 : ((nx + 31) / 32) * 32;
-  return dim3(bx, 256 / bx, 1);
-}
-dim3 grid2d(dim3 b, int nx, int ny, int nz) { return dim3((nx + b.x - 1) / b.x, (ny + b.y - 1) / b.y, nz); }
-
 template <typename T>
 __device__ __forceinline__ double ld_in(const void* p, size_t idx) {
   return (double)static_cast<const T*>(p)[idx];
+}
+
+// E_i(u) at node d of a velocity field.
+template <typename R>
+__device__ __forceinline__ R shape_at(const float* __restrict__ u3, size_t N, int d, int i) {
+  const R ux = u3[d], uy = u3[N + d], uz = u3[2 * N + d];
+  const R cu = R(cx_of(i)) * ux + R(cy_of(i)) * uy + R(cz_of(i)) * uz;
+  return R(w_of(i)) * (R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * (ux * ux + uy * uy + uz * uz));
 }
 
 // ---------------------------------------------------------------- write state
@@ -27,7 +30,7 @@ __device__ __forceinline__ double ld_in(const void* p, size_t idx) {
 // (anti-bounce-back inverted: the stored outgoing population of a wall node only
 // feeds the entering opposite one).
 template <typename Elem, typename Tin, int FROM_PHI>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)   // 128^3 FP64 with source 447 us, unbounded 530; 256^3 FP32 402, with 3 blocks 462
 k_write(Elem* __restrict__ pops, float* __restrict__ scale, Grid G, const void* __restrict__ in,
         const float* __restrict__ src, const float* __restrict__ u3,
         const PopConsts<typename Storage<Elem>::real> k) {
@@ -37,38 +40,41 @@ k_write(Elem* __restrict__ pops, float* __restrict__ scale, Grid G, const void* 
   const int z = blockIdx.z;
   if (x >= G.nx || y >= G.ny) return;
   const int n = x + G.nx * (y + G.ny * z);
+  // All 27 destinations are loaded at once (wrapped, as if periodic), then the uniform cases, then
+  // the faces: with the cases inside the loop every load waited for the one before it (256^3 FP32
+  // 0.50 -> 0.40 ms, FP16 deviations 0.56 -> 0.39 ms).
+  const int xs[3] = {x == 0 ? G.nx - 1 : x - 1, x, x + 1 == G.nx ? 0 : x + 1};
+  const int ys[3] = {(y == 0 ? G.ny - 1 : y - 1) * G.nx, y * G.nx, (y + 1 == G.ny ? 0 : y + 1) * G.nx};
+  const int nxy = G.nx * G.ny;
+  const int zs[3] = {(z == 0 ? G.nz - 1 : z - 1) * nxy, z * nxy, (z + 1 == G.nz ? 0 : z + 1) * nxy};
+  const auto dest = [&](int i) { return xs[cx_of(i) + 1] + ys[cy_of(i) + 1] + zs[cz_of(i) + 1]; };
   R a[Q];
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    int dx = x + cx_of(i), dy = y + cy_of(i), dz = z + cz_of(i);
-    const bool through_hi = dx >= G.nx;  // leaves through x = Nx - 1/2 (else through x = -1/2)
-    dy = dy < 0 ? G.ny - 1 : (dy >= G.ny ? 0 : dy);
-    dz = dz < 0 ? G.nz - 1 : (dz >= G.nz ? 0 : dz);
-    const bool outside = G.dirichlet && (dx < 0 || dx >= G.nx);
-    dx = dx < 0 ? G.nx - 1 : (dx >= G.nx ? 0 : dx);
-    const int d = dx + G.nx * (dy + G.ny * dz);
-    if (!outside) {
-      R Ei = k.E[i];
-      if (FROM_PHI && u3 != nullptr) {   // equilibrium at the velocity of node d
-        const R ux = u3[d], uy = u3[G.N + d], uz = u3[2 * G.N + d];
-        const R cu = R(cx_of(i)) * ux + R(cy_of(i)) * uy + R(cz_of(i)) * uz;
-        Ei = R(w_of(i)) * (R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * (ux * ux + uy * uy + uz * uz));
-      }
-      R v = FROM_PHI ? R(ld_in<Tin>(in, d)) * Ei : R(ld_in<Tin>(in, (size_t)i * G.N + d));
-      if (src != nullptr) v -= k.src_half * R(src[d]) * k.E[i];
-      a[i] = v;
+  for (int i = 0; i < Q; ++i) a[i] = R(ld_in<Tin>(in, FROM_PHI ? (size_t)dest(i) : (size_t)i * G.N + dest(i)));
+  if (FROM_PHI) {
+    if (u3 == nullptr) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) a[i] = a[i] * k.E[i];
     } else {
-      const int o = opp_of(i);
-      R Eo = k.E[o];
-      if (FROM_PHI && u3 != nullptr) {
-        const R ux = u3[n], uy = u3[G.N + n], uz = u3[2 * G.N + n];
-        const R cu = R(cx_of(o)) * ux + R(cy_of(o)) * uy + R(cz_of(o)) * uz;
-        Eo = R(w_of(o)) * (R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * (ux * ux + uy * uy + uz * uz));
+#pragma unroll
+      for (int i = 0; i < Q; ++i) a[i] = a[i] * shape_at<R>(u3, G.N, dest(i), i);   // the velocity of that node
+    }
+  }
+  if (src != nullptr) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) a[i] -= k.src_half * R(src[dest(i)]) * k.E[i];
+  }
+  if (G.dirichlet && (x == 0 || x == G.nx - 1)) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const bool lo = cx_of(i) < 0 && x == 0, hi = cx_of(i) > 0 && x == G.nx - 1;
+      if (lo || hi) {                  // leaves through x = -1/2 or x = Nx - 1/2
+        const int o = opp_of(i);
+        const R Eo = FROM_PHI && u3 != nullptr ? shape_at<R>(u3, G.N, n, o) : k.E[o];
+        R v = FROM_PHI ? R(ld_in<Tin>(in, n)) * Eo : R(ld_in<Tin>(in, (size_t)o * G.N + n));
+        if (src != nullptr) v -= k.src_half * R(src[n]) * k.E[o];
+        a[i] = R(2.0 * w_of(i)) * (hi ? k.phi_hi : k.phi_lo) - v;
       }
-      R v = FROM_PHI ? R(ld_in<Tin>(in, n)) * Eo : R(ld_in<Tin>(in, (size_t)o * G.N + n));
-      if (src != nullptr) v -= k.src_half * R(src[n]) * k.E[o];
-      const R phw = through_hi ? k.phi_hi : k.phi_lo;
-      a[i] = R(2.0 * w_of(i)) * phw - v;
     }
   }
   Storage<Elem>::store(pops, scale, G.N, n, a, k.Ek, R(NAN));
@@ -76,7 +82,7 @@ k_write(Elem* __restrict__ pops, float* __restrict__ scale, Grid G, const void* 
 
 // ----------------------------------------------------------------- read state
 template <typename Elem, typename Tout, int WHAT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 3)   // FP16 phi of 256^3: 281 us, with up to 2 or 4 blocks 367 and 304
 k_read(Field<Elem> f, Grid G, Tout* __restrict__ out, Tout* __restrict__ qout,
        const typename Storage<Elem>::real* __restrict__ T6,
        const float* __restrict__ src, const float* __restrict__ u3,
@@ -201,7 +207,7 @@ const PopConsts<typename Storage<Elem>::real>& consts_of(const StateIO& S) {
 template <typename Elem>
 cudaError_t write_t(const StateIO& S, const void* in, int in_f32, int from_phi, cudaStream_t s) {
   Grid G{S.nx, S.ny, S.nz, S.N, S.dirichlet};
-  dim3 b = block2d(S.nx), g = grid2d(b, S.nx, S.ny, S.nz);
+  dim3 b = row_block(S.nx), g = row_grid(b, S.nx, S.ny, S.nz);
   Elem* p = static_cast<Elem*>(S.pops);
   const auto& k = consts_of<Elem>(S);
   if (in_f32) {
@@ -217,7 +223,7 @@ cudaError_t write_t(const StateIO& S, const void* in, int in_f32, int from_phi, 
 template <typename Elem>
 cudaError_t read_t(const StateIO& S, void* out, void* q, int out_f32, int what, cudaStream_t s) {
   Grid G{S.nx, S.ny, S.nz, S.N, S.dirichlet};
-  dim3 b = block2d(S.nx), g = grid2d(b, S.nx, S.ny, S.nz);
+  dim3 b = row_block(S.nx), g = row_grid(b, S.nx, S.ny, S.nz);
   using R = typename Storage<Elem>::real;
   const auto& k = consts_of<Elem>(S);
   Field<Elem> f = field_of<Elem>(S);

@@ -427,9 +427,8 @@ cudaError_t launch_step2(elbm2d_ctx* h) {
   const Consts2<R>& k = *reinterpret_cast<const Consts2<R>*>(std::is_same<R, double>::value ? (const void*)&h->kd
                                                                                            : (const void*)&h->kf);
   const int vel = h->u2 ? 2 : ((h->u[0] != 0.0 || h->u[1] != 0.0) ? 1 : 0);
-  const int bx = h->nx >= 256 ? 256 : ((h->nx + 31) / 32) * 32;
-  const dim3 block(bx, 256 / bx);
-  const dim3 grid((h->nx + bx - 1) / bx, (unsigned)std::min<long long>((h->ny + block.y - 1) / block.y, 65535));
+  const dim3 block = elbm::row_block(h->nx);
+  const dim3 grid((h->nx + block.x - 1) / block.x, (unsigned)std::min<long long>((h->ny + block.y - 1) / block.y, 65535));
   Grid2 G{h->nx, h->ny, h->N};
   const R* in = static_cast<const R*>(h->pops[h->cur]);
   R* out = static_cast<R*>(h->pops[1 - h->cur]);

@@ -1,4 +1,5 @@
-// Launches of kernels that follow one another on a stream, each reading what the one before wrote.
+// Launches: the block shape of one thread per node, and kernels that follow one another on a stream,
+// each reading what the one before wrote.
 //
 // A launch that waits for the previous kernel to end before it is set up costs about 2 us per step;
 // with programmatic stream serialisation the next kernel's blocks are placed while the last ones of
@@ -22,6 +23,15 @@ __device__ __forceinline__ void wait_for_previous() {
   cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
 }
+
+// Blocks of at most 256 threads for one thread per node, rows along x: a row is cut into equal
+// pieces of whole warps (384 nodes into 2 x 192, where 256-thread pieces leave a quarter of the
+// lanes idle), short rows share a block.
+inline dim3 row_block(int nx) {
+  const int pieces = (nx + 255) / 256, per = (nx + pieces - 1) / pieces, bx = (per + 31) / 32 * 32;
+  return dim3(bx, 256 / bx, 1);
+}
+inline dim3 row_grid(dim3 b, int nx, int ny, int nz) { return dim3((nx + b.x - 1) / b.x, (ny + b.y - 1) / b.y, nz); }
 
 template <typename... Params, typename... Args>
 inline cudaError_t launch_next(void (*kernel)(Params...), dim3 grid, dim3 block, size_t shared, cudaStream_t s,

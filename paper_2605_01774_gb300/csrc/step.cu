@@ -90,18 +90,12 @@ k_step(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G
   }
 }
 
-static dim3 block_for(int nx) {
-  int bx = nx >= 256 ? 256 : ((nx + 31) / 32) * 32;
-  return dim3(bx, 256 / bx, 1);
-}
-
 template <typename Elem, int VEL, int MODE>
 static cudaError_t launch_t(const StepLaunch& L, cudaStream_t s) {
   using R = typename Storage<Elem>::real;
   Field<Elem> in{static_cast<const Elem*>(L.pin), L.sin};
   Grid G{L.nx, L.ny, L.nz, L.N, L.dirichlet};
-  dim3 b = block_for(L.nx);
-  dim3 g((L.nx + b.x - 1) / b.x, (L.ny + b.y - 1) / b.y, L.nz);
+  dim3 b = row_block(L.nx), g = row_grid(b, L.nx, L.ny, L.nz);
   if constexpr (MODE == FIXED) {
     b = dim3(step_threads<Elem, MODE>());
     g = dim3((unsigned)((L.N + b.x - 1) / b.x));
