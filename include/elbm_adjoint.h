@@ -12,7 +12,9 @@
  *
  * Misfit: J = 1/2 sum_{t in obs} sum_x (phi_t(x) - phi*_t(x))^2 with phi_t the
  * zeroth moment after t steps.  The gradient is computed by a reverse sweep over
- * checkpoints taken every K steps, recomputing each K-step segment forward.
+ * checkpoints taken every K steps, recomputing each K-step segment forward; runs whose
+ * states fit 4 GiB keep them all and recompute nothing.  The handle keeps up to 4 GiB of
+ * states between calls.
  *
  * Arrays are device pointers in the handle's precision (double for ELBM_F64,
  * float for ELBM_F32), layout [component][N] with node n = x + Nx (y + Ny z).

@@ -24,11 +24,24 @@
 
 #include "../../include/elbm.h"
 #include "../../include/elbm_adjoint.h"
+#include "collide64.cuh"
 #include "internal.h"
+#include "launch.cuh"
 
 using namespace elbm;
 
 namespace {
+
+// Threads per block of the step kernels.  FP64: 30 x 32 x 28 nodes are 105 blocks of 256 threads,
+// fewer than SMs; blocks of 64 put the same warps on all of them.
+template <typename R>
+constexpr int STEP_THREADS = sizeof(R) == 8 ? 64 : 128;
+
+// States of a run that are kept rather than recomputed, and the workspace that a handle keeps
+// between calls (a larger one is given back at the end of the call).  64^3 FP32 with 32 steps and
+// checkpoints every 8 (3.1 ms a call) recomputed 28 of them, 14 us each, and got and returned 0.4 GB
+// on each call.
+constexpr size_t KEEP_BYTES = 4ull << 30;
 
 struct AGrid {
   int nx, ny, nz;
@@ -52,25 +65,58 @@ __device__ __forceinline__ int nb(const AGrid& G, int x, int y, int z, int dx, i
   return x + G.nx * (y + G.ny * z);
 }
 
+// sum_i c_i v_i, taken three populations (cz = -1, 0, 1 of one (cx, cy)) at a time.
 template <typename R>
-__device__ __forceinline__ R cdot(int i, R vx, R vy, R vz) {
-  return R(cx_of(i)) * vx + R(cy_of(i)) * vy + R(cz_of(i)) * vz;
-}
+struct FirstMoment {
+  R x = R(0), y = R(0), z = R(0);
+  __device__ __forceinline__ void add(int p, R v0, R v1, R v2) {
+    const int cx = p / 3 - 1, cy = p % 3 - 1;
+    z += v2 - v0;
+    const R s = v0 + v1 + v2;
+    if (cy != 0) y = cy > 0 ? y + s : y - s;
+    if (cx != 0) x = cx > 0 ? x + s : x - s;
+  }
+};
+
+// c_i . v for all 27 velocities, as (cx vx + cy vy) + cz vz: the order in which den and its guard
+// have always been rounded, so that the same nodes are stabilised.
+template <typename R>
+struct DotsXYZ {
+  R d[Q];
+  __device__ __forceinline__ DotsXYZ(R vx, R vy, R vz) {
+#pragma unroll
+    for (int p = 0; p < 9; ++p) {
+      const int cx = p / 3 - 1, cy = p % 3 - 1;
+      const R x = cx == 0 ? R(0) : (cx > 0 ? vx : -vx);
+      const R xy = cy == 0 ? x : (cx == 0 ? (cy > 0 ? vy : -vy) : (cy > 0 ? x + vy : x - vy));
+      d[3 * p] = p == 4 ? -vz : xy - vz;
+      d[3 * p + 1] = xy;
+      d[3 * p + 2] = p == 4 ? vz : xy + vz;
+    }
+  }
+};
 
 // ---------------------------------------------------------------- parameters -> T
+// What dL/dtheta needs besides T is kept: aux[12][N] holds sin and cos of a, b, c, then t_k, then
+// dt_k / d ln d_k.
 template <typename R>
-__global__ void k_params_to_T(const R* __restrict__ th, R* __restrict__ T6, int N) {
+__global__ void k_params_to_T(const R* __restrict__ th, R* __restrict__ T6, double* __restrict__ aux, int N) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
+  const size_t S = N;
   double t[3];
   for (int k = 0; k < 3; ++k) {
-    const double d = exp((double)th[k * N + n]);
-    t[k] = 12.0 * d / (1.0 + 6.0 * d);
+    const double d = exp((double)th[k * N + n]), r = 1.0 / (1.0 + 6.0 * d);
+    t[k] = 12.0 * d * r;
+    aux[(6 + k) * S + n] = t[k];
+    aux[(9 + k) * S + n] = t[k] * r;
   }
   double sa, ca, sb, cb, sc, cc;
   sincos((double)th[3 * N + n], &sa, &ca);
   sincos((double)th[4 * N + n], &sb, &cb);
   sincos((double)th[5 * N + n], &sc, &cc);
+  const double v[6] = {sa, ca, sb, cb, sc, cc};
+  for (int q = 0; q < 6; ++q) aux[q * S + n] = v[q];
   const double Rm[3][3] = {{ca * cb * cc - sa * sc, -ca * cb * sc - sa * cc, ca * sb},
                            {sa * cb * cc + ca * sc, -sa * cb * sc + ca * cc, sa * sb},
                            {-sb * cc, sb * sc, cb}};
@@ -83,69 +129,51 @@ __global__ void k_params_to_T(const R* __restrict__ th, R* __restrict__ T6, int 
 }
 
 // dL/dtheta from the accumulated dL/dT (6 unique components, off-diagonals counted once).
+// With G the symmetric full-matrix gradient and H = R^T G R (the principal frame):
+// dL/dt_k = H_kk, and turning the frame by dw about its own axes changes T by R [dw]x diag(t) R^T
+// plus its transpose, so dL/dw_x = 2 (t_y - t_z) H_yz and cyclic.  The angles turn it about
+//   c: its z axis;  b: (sin c, cos c, 0);  a: the third row of R.
+// FP64 issues at 1/64 of the FP32 rate, so the sines, exponentials and quotients are not repeated
+// here (64^3 FP32: 221 -> 49 us).
 template <typename R>
-__global__ void k_Tbar_to_params(const R* __restrict__ th, const double* __restrict__ Tbar, R* __restrict__ gth,
-                                 int N) {
+__global__ void k_Tbar_to_params(const double* __restrict__ aux, const double* __restrict__ Tbar,
+                                 R* __restrict__ gth, int N) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
-  double d[3], t[3], dt[3];
+  const size_t S = N;
+  const double sa = aux[n], ca = aux[S + n], sb = aux[2 * S + n], cb = aux[3 * S + n], sc = aux[4 * S + n],
+               cc = aux[5 * S + n];
+  const double t[3] = {aux[6 * S + n], aux[7 * S + n], aux[8 * S + n]};
+  const double Gm[6] = {Tbar[n],           0.5 * Tbar[S + n],     0.5 * Tbar[2 * S + n],
+                        Tbar[3 * S + n],   0.5 * Tbar[4 * S + n], Tbar[5 * S + n]};
+  const double cbcc = cb * cc, cbsc = cb * sc;
+  // columns of R
+  const double q[3][3] = {{ca * cbcc - sa * sc, sa * cbcc + ca * sc, -sb * cc},
+                          {-ca * cbsc - sa * cc, -sa * cbsc + ca * cc, sb * sc},
+                          {ca * sb, sa * sb, cb}};
+  double w[3][3];   // G times the columns
+#pragma unroll
   for (int k = 0; k < 3; ++k) {
-    d[k] = exp((double)th[k * N + n]);
-    t[k] = 12.0 * d[k] / (1.0 + 6.0 * d[k]);
-    dt[k] = 12.0 * d[k] / ((1.0 + 6.0 * d[k]) * (1.0 + 6.0 * d[k]));  // dt_k / d ln d_k
+    w[k][0] = Gm[0] * q[k][0] + Gm[1] * q[k][1] + Gm[2] * q[k][2];
+    w[k][1] = Gm[1] * q[k][0] + Gm[3] * q[k][1] + Gm[4] * q[k][2];
+    w[k][2] = Gm[2] * q[k][0] + Gm[4] * q[k][1] + Gm[5] * q[k][2];
   }
-  // symmetric full-matrix gradient: diagonal as is, off-diagonal halves
-  const double g6[6] = {Tbar[n], Tbar[N + n], Tbar[2 * N + n], Tbar[3 * N + n], Tbar[4 * N + n], Tbar[5 * N + n]};
-  const double Gm[3][3] = {{g6[0], 0.5 * g6[1], 0.5 * g6[2]},
-                           {0.5 * g6[1], g6[3], 0.5 * g6[4]},
-                           {0.5 * g6[2], 0.5 * g6[4], g6[5]}};
-  const double a = th[3 * N + n], b = th[4 * N + n], c = th[5 * N + n];
-  const double sa = sin(a), ca = cos(a), sb = sin(b), cb = cos(b), sc = sin(c), cc = cos(c);
-  const double Rz_a[3][3] = {{ca, -sa, 0}, {sa, ca, 0}, {0, 0, 1}};
-  const double dRz_a[3][3] = {{-sa, -ca, 0}, {ca, -sa, 0}, {0, 0, 0}};
-  const double Ry_b[3][3] = {{cb, 0, sb}, {0, 1, 0}, {-sb, 0, cb}};
-  const double dRy_b[3][3] = {{-sb, 0, cb}, {0, 0, 0}, {-cb, 0, -sb}};
-  const double Rz_c[3][3] = {{cc, -sc, 0}, {sc, cc, 0}, {0, 0, 1}};
-  const double dRz_c[3][3] = {{-sc, -cc, 0}, {cc, -sc, 0}, {0, 0, 0}};
-  auto mul = [](const double A[3][3], const double B[3][3], double C[3][3]) {
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) {
-        double s = 0;
-        for (int k = 0; k < 3; ++k) s += A[i][k] * B[k][j];
-        C[i][j] = s;
-      }
-  };
-  double tmp[3][3], Q[3][3], dQa[3][3], dQb[3][3], dQc[3][3];
-  mul(Rz_a, Ry_b, tmp);
-  mul(tmp, Rz_c, Q);
-  mul(dRz_a, Ry_b, tmp);
-  mul(tmp, Rz_c, dQa);
-  mul(Rz_a, dRy_b, tmp);
-  mul(tmp, Rz_c, dQb);
-  mul(Rz_a, Ry_b, tmp);
-  mul(tmp, dRz_c, dQc);
-  // dL/dt_k = (Q^T G Q)_kk ; dL/dangle = sum_ab [2 G Q Lambda]_ab dQ_ab
-  double GQ[3][3];
-  mul(Gm, Q, GQ);
-  for (int k = 0; k < 3; ++k) {
-    double s = 0;
-    for (int i = 0; i < 3; ++i) s += Q[i][k] * GQ[i][k];
-    gth[k * N + n] = (R)(s * dt[k]);
-  }
-  const double(*dQ[3])[3] = {dQa, dQb, dQc};
-  for (int m = 0; m < 3; ++m) {
-    double s = 0;
-    for (int i = 0; i < 3; ++i)
-      for (int k = 0; k < 3; ++k) s += 2.0 * GQ[i][k] * t[k] * dQ[m][i][k];
-    gth[(3 + m) * N + n] = (R)s;
-  }
+  const auto H = [&](int i, int k) { return q[i][0] * w[k][0] + q[i][1] * w[k][1] + q[i][2] * w[k][2]; };
+#pragma unroll
+  for (int k = 0; k < 3; ++k) gth[k * N + n] = (R)(H(k, k) * aux[(9 + k) * S + n]);
+  const double wx = 2.0 * (t[1] - t[2]) * H(1, 2), wy = 2.0 * (t[2] - t[0]) * H(2, 0), wz = 2.0 * (t[0] - t[1]) * H(0, 1);
+  gth[3 * N + n] = (R)(q[0][2] * wx + q[1][2] * wy + cb * wz);
+  gth[4 * N + n] = (R)(sc * wx + cc * wy);
+  gth[5 * N + n] = (R)wz;
 }
 
 // ---------------------------------------------------------------- forward (push)
+// States are read with plain loads: the kernel may be resident while the one before it still writes
+// them (launch.cuh).
 template <typename R>
-__global__ void __launch_bounds__(256)
-k_adj_forward(const R* __restrict__ Gin, R* __restrict__ Gout, const R* __restrict__ T6, AGrid G,
-              const PopConsts<R> k, unsigned long long* fb) {
+__global__ void __launch_bounds__(STEP_THREADS<R>)
+k_adj_forward(const R* Gin, R* Gout, const R* __restrict__ T6, AGrid G, const PopConsts<R> k, unsigned long long* fb) {
+  wait_for_previous();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   bool took = false;
   if (n < G.N) {
@@ -164,14 +192,63 @@ k_adj_forward(const R* __restrict__ Gin, R* __restrict__ Gout, const R* __restri
   if (m && (threadIdx.x & 31) == 0) atomicAdd(fb, (unsigned long long)__popc(m));
 }
 
+// One of the few nodes that fixed point cannot hold, out of line.
+__device__ __noinline__ bool adj_node_f64(const double* Gin, double* Gout, const double* T6, const AGrid& G, int n,
+                                          const PopConsts<double>& k) {
+  double g[Q], phi;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) g[i] = Gin[i * G.N + n];
+  const Sym6<double> T{T6[n], T6[G.N + n], T6[2 * G.N + n], T6[3 * G.N + n], T6[4 * G.N + n], T6[5 * G.N + n]};
+  const bool took = collide_node<double, 1>(g, T, k, true, phi);
+  int x, y, z;
+  coords(G, n, x, y, z);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) Gout[i * G.N + nb(G, x, y, z, cx_of(i), cy_of(i), cz_of(i))] = g[i];
+  return took;
+}
+
+// The FP64 step with the fixed-point collision (fixed.cuh) that the lattice's own steps use:
+// 30 x 32 x 28 nodes 34 -> 15.6 us a launch.
+struct FixedStep {
+  FixConsts fix;
+  PopConsts<double> pop;
+};
+__global__ void __launch_bounds__(64, 6)
+k_adj_forward_fixed(const double* Gin, double* Gout, const double* __restrict__ T6, const __grid_constant__ AGrid G,
+                    const __grid_constant__ FixedStep c, unsigned long long* fb) {
+  __shared__ int64_t kept[KEPT * 64];
+  wait_for_previous();
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  bool took = false;
+  if (n < G.N) {
+    double g[Q], T[6];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] = Gin[i * G.N + n];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) T[q] = T6[q * G.N + n];
+    int x, y, z;
+    coords(G, n, x, y, z);
+    InShared<64> keep{kept + threadIdx.x};
+    if (!collide_fixed<1>(g, T, 0.0, false, true, c.fix, keep, took,
+                          [&](int i, double v) { Gout[i * G.N + nb(G, x, y, z, cx_of(i), cy_of(i), cz_of(i))] = v; }))
+      took = adj_node_f64(Gin, Gout, T6, G, n, c.pop);
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, took);
+  if (m && (threadIdx.x & 31) == 0) atomicAdd(fb, (unsigned long long)__popc(m));
+}
+
 // ---------------------------------------------------------------- one-step VJP
-// Gbar_out(y) = J^T gathered adjoint; Tbar(y) += dL/dT (FP64 accumulators); if target
-// is given (an observation time), Gbar_out(y)_i += phi(y) - target(y).
+// Gbar_out(y) = J^T gathered adjoint; Tbar(y) = or += dL/dT (FP64 accumulators; `first` sets them);
+// if target is given (an observation time), Gbar_out(y)_i += phi(y) - target(y).
+// Bound by instruction issue (FP64: by its pipe), so c_i is never multiplied by: products c_i . v
+// come from shared partial sums (DotsXYZ), sums over c_i v_i go by threes (FirstMoment), and dh_i is
+// kept for the second pass: about 800 operations per node (were 1450; with the blocks of STEP_THREADS
+// a launch for 64^3 FP32 takes 28 -> 22 us, FP64 30 x 32 x 28 94 -> 60 us).
 template <typename R>
-__global__ void __launch_bounds__(256)
-k_adj_vjp(const R* __restrict__ Gn, const R* __restrict__ Gbar_next, R* __restrict__ Gbar_out,
-          const R* __restrict__ T6, double* __restrict__ Tbar, const R* __restrict__ target, AGrid G,
-          const PopConsts<R> k) {
+__global__ void __launch_bounds__(STEP_THREADS<R>, sizeof(R) == 4 ? 4 : 1)   // 64^3 FP32, whole call: 1.37, 1.21, 1.18 ms with 1, 3, 4
+k_adj_vjp(const R* Gn, const R* Gbar_next, R* Gbar_out, const R* __restrict__ T6, double* Tbar,
+          const R* __restrict__ target, AGrid G, const PopConsts<R> k, int first) {
+  wait_for_previous();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= G.N) return;
   int x, y, z;
@@ -190,71 +267,81 @@ k_adj_vjp(const R* __restrict__ Gn, const R* __restrict__ Gbar_next, R* __restri
   R tx, ty, tz;
   sym_mul(T, jx, jy, jz, tx, ty, tz);
   const R ax = tx - jx, ay = ty - jy, az = tz - jz;
-  R kappa = R(0), num = R(0), den = R(0), inv = R(0);
-  const R tiny = sizeof(R) == 4 ? R(1e-30) : R(1e-300);
-  const bool kap_on_phi = phi > tiny;
-  if (kap_on_phi) {
-    inv = R(1) / phi;
+  // ---- reverse of g* = psi E - kappa g + 3 W c.b, psi = (1 + kappa) phi, b = a + kappa j
+  R psib = R(0), kapb = R(0);
+  FirstMoment<R> bb;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const R dh = g[i] * inv - k.E[i] - R(3.0 * w_of(i)) * cdot<R>(i, jx * inv, jy * inv, jz * inv);
-      num += dh * (k.K3[i] * cdot<R>(i, ax * inv, ay * inv, az * inv) + k.L[i]);
-      den += dh * dh * k.M[i];
+  for (int p = 0; p < 9; ++p) {
+    R w3[3];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const int i = 3 * p + m;
+      psib += yb[i] * k.E[i];
+      kapb -= yb[i] * g[i];
+      w3[m] = R(3.0 * w_of(i)) * yb[i];
     }
+    bb.add(p, w3[0], w3[1], w3[2]);
   }
-  const bool kap_on = kap_on_phi && den > k.theta2;
-  if (kap_on) kappa = num / den;
-  // ---- reverse
-  R psib = R(0), kapb = R(0), bbx = R(0), bby = R(0), bbz = R(0);
-  R gb[Q];
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    psib += yb[i] * k.E[i];
-    kapb -= yb[i] * g[i];
-    gb[i] = -kappa * yb[i];
-    const R w3 = R(3.0 * w_of(i)) * yb[i];
-    bbx += R(cx_of(i)) * w3;
-    bby += R(cy_of(i)) * w3;
-    bbz += R(cz_of(i)) * w3;
-  }
-  // psi = (1 + kappa) phi ; b = a + kappa j
   kapb += psib * phi;
-  R phib = psib * (R(1) + kappa);
-  R abx = bbx, aby = bby, abz = bbz;
-  kapb += bbx * jx + bby * jy + bbz * jz;
-  R jbx = kappa * bbx, jby = kappa * bby, jbz = kappa * bbz;
-  if (kap_on) {
-    const R numb = kapb / den;
-    const R denb = -kapb * kappa / den;
-    R apbx = R(0), apby = R(0), apbz = R(0), jpbx = R(0), jpby = R(0), jpbz = R(0), invb = R(0);
+  kapb += bb.x * jx + bb.y * jy + bb.z * jz;
+  R kappa = R(0);
+  R phib = R(0);
+  R abx = bb.x, aby = bb.y, abz = bb.z, jbx = R(0), jby = R(0), jbz = R(0);
+  const R tiny = sizeof(R) == 4 ? R(1e-30) : R(1e-300);
+  bool on = false;
+  if (phi > tiny) {
+    const R inv = R(1) / phi;
+    R dh[Q];
+    R num = R(0), den = R(0);
+    const DotsXYZ<R> ca(ax * inv, ay * inv, az * inv);
+    {
+      const DotsXYZ<R> cj(jx * inv, jy * inv, jz * inv);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const R cj = cdot<R>(i, jx * inv, jy * inv, jz * inv);
-      const R ca = cdot<R>(i, ax * inv, ay * inv, az * inv);
-      const R dh = g[i] * inv - k.E[i] - R(3.0 * w_of(i)) * cj;
-      const R t = k.K3[i] * ca + k.L[i];
-      const R dhb = numb * t + R(2) * denb * dh * k.M[i];
-      const R cak = numb * dh * k.K3[i];            // d num / d (c_i . a')
-      apbx += R(cx_of(i)) * cak;
-      apby += R(cy_of(i)) * cak;
-      apbz += R(cz_of(i)) * cak;
-      gb[i] += dhb * inv;
-      invb += dhb * g[i];
-      const R cjb = -dhb * R(3.0 * w_of(i));        // d / d (c_i . j')
-      jpbx += R(cx_of(i)) * cjb;
-      jpby += R(cy_of(i)) * cjb;
-      jpbz += R(cz_of(i)) * cjb;
+      for (int i = 0; i < Q; ++i) {
+        dh[i] = g[i] * inv - k.E[i] - R(3.0 * w_of(i)) * cj.d[i];
+        num += dh[i] * (k.K3[i] * ca.d[i] + k.L[i]);
+        den += dh[i] * dh[i] * k.M[i];
+      }
     }
-    // a' = a inv ; j' = j inv ; inv = 1 / phi
-    abx += apbx * inv;
-    aby += apby * inv;
-    abz += apbz * inv;
-    invb += apbx * ax + apby * ay + apbz * az;
-    jbx += jpbx * inv;
-    jby += jpby * inv;
-    jbz += jpbz * inv;
-    invb += jpbx * jx + jpby * jy + jpbz * jz;
-    phib -= invb * inv * inv;
+    on = den > k.theta2;
+    if (on) {
+      kappa = num / den;
+      const R numb = kapb / den;
+      const R denb2 = R(-2) * numb * kappa;            // twice d/d den
+      R invb = R(0);
+      FirstMoment<R> apb, jpb;                         // a' = a inv, j' = j inv, inv = 1 / phi
+#pragma unroll
+      for (int p = 0; p < 9; ++p) {
+        R cak[3], cjb[3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          const int i = 3 * p + m;
+          const R t = k.K3[i] * ca.d[i] + k.L[i];
+          const R dhb = numb * t + denb2 * (dh[i] * k.M[i]);
+          cak[m] = dh[i] * k.K3[i];                    // d num / d (c_i . a'), times numb below
+          cjb[m] = R(3.0 * w_of(i)) * dhb;             // -d / d (c_i . j')
+          yb[i] = dhb * inv - kappa * yb[i];
+          invb += dhb * g[i];
+        }
+        apb.add(p, cak[0], cak[1], cak[2]);
+        jpb.add(p, cjb[0], cjb[1], cjb[2]);
+      }
+      const R apx = numb * apb.x, apy = numb * apb.y, apz = numb * apb.z;
+      abx += apx * inv;
+      aby += apy * inv;
+      abz += apz * inv;
+      invb += apx * ax + apy * ay + apz * az;
+      jbx = kappa * bb.x - jpb.x * inv;
+      jby = kappa * bb.y - jpb.y * inv;
+      jbz = kappa * bb.z - jpb.z * inv;
+      invb -= jpb.x * jx + jpb.y * jy + jpb.z * jz;
+      phib = psib * (R(1) + kappa) - invb * inv * inv;
+    }
+  }
+  if (!on) {                                           // kappa = 0
+    phib = psib;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) yb[i] = R(0);
   }
   // a = T j - j
   R Tax, Tay, Taz;
@@ -262,19 +349,21 @@ k_adj_vjp(const R* __restrict__ Gn, const R* __restrict__ Gbar_next, R* __restri
   jbx += Tax - abx;
   jby += Tay - aby;
   jbz += Taz - abz;
-  Tbar[n] += (double)(abx * jx);
-  Tbar[G.N + n] += (double)(abx * jy + aby * jx);
-  Tbar[2 * G.N + n] += (double)(abx * jz + abz * jx);
-  Tbar[3 * G.N + n] += (double)(aby * jy);
-  Tbar[4 * G.N + n] += (double)(aby * jz + abz * jy);
-  Tbar[5 * G.N + n] += (double)(abz * jz);
+  const R tb[6] = {abx * jx, abx * jy + aby * jx, abx * jz + abz * jx, aby * jy, aby * jz + abz * jy, abz * jz};
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    // one writer per node: an addition without a returned value only keeps the sum off the thread's
+    // path (64^3 FP32, 32 steps: 1.43 -> 1.21 ms a call)
+    double* const acc = Tbar + q * (size_t)G.N + n;
+    if (first) *acc = (double)tb[q];
+    else atomicAdd(acc, (double)tb[q]);
+  }
   // j = m - phi u ; m = sum c g ; phi = sum g
   phib -= k.ux * jbx + k.uy * jby + k.uz * jbz;
-  R inj = R(0);
-  if (target != nullptr) inj = phi - target[n];
+  if (target != nullptr) phib += phi - target[n];
+  const DotsXYZ<R> cjb(jbx, jby, jbz);
 #pragma unroll
-  for (int i = 0; i < Q; ++i)
-    Gbar_out[i * G.N + n] = gb[i] + R(cx_of(i)) * jbx + R(cy_of(i)) * jby + R(cz_of(i)) * jbz + phib + inj;
+  for (int i = 0; i < Q; ++i) Gbar_out[i * G.N + n] = yb[i] + (cjb.d[i] + phib);
 }
 
 // misfit contribution 1/2 sum (phi - target)^2 and phi-adjoint seed at the last step
@@ -293,7 +382,7 @@ k_adj_misfit(const R* __restrict__ Gs, const R* __restrict__ target, double* __r
     v = 0.5 * d * d;
     if (seed != nullptr) {
 #pragma unroll
-      for (int i = 0; i < Q; ++i) seed[i * N + n] += (R)d;
+      for (int i = 0; i < Q; ++i) seed[i * N + n] = (R)d;
     }
   }
   sm[threadIdx.x] = v;
@@ -318,8 +407,10 @@ struct elbm_adjoint_ctx {
   PopConsts<float> kf{};
   void* T6 = nullptr;              // [6][N] R
   double* Tbar = nullptr;          // [6][N]
-  void* ck = nullptr;              // checkpoints, allocated per run
-  void* seg = nullptr;             // segment states
+  FixedStep fixed{};               // FP64 steps in fixed point
+  double* aux = nullptr;           // [12][N] (k_params_to_T)
+  void* states = nullptr;          // checkpoints and segment states
+  size_t state_bytes = 0;
   void* gbar[2] = {nullptr, nullptr};
   double* part = nullptr;
   unsigned long long* fb = nullptr;
@@ -369,6 +460,8 @@ void consts_for(elbm_adjoint_ctx* h) {
   f.uz = (float)u[2];
   f.theta2 = (float)k.theta2;
   f.eps = 0.f;
+  h->fixed.fix = fix_consts(h->kd);
+  h->fixed.pop = h->kd;
 }
 
 template <typename R>
@@ -393,48 +486,117 @@ __global__ void k_adj_init(const R* __restrict__ phi0, R* __restrict__ Gs, int N
   for (int i = 0; i < Q; ++i) Gs[i * N + n] = p * k.E[i];
 }
 
+int step_blocks(int N, int threads) { return (N + threads - 1) / threads; }
+
+// One forward step (fallback nodes counted in *fb).
 template <typename R>
-elbm_status run_t(elbm_adjoint_ctx* h, const R* theta, const R* phi0, int64_t nsteps, int nobs, const int64_t* obs,
-                  const R* targets, double* J, R* grad, int64_t* nfb) {
-  const AGrid G = h->G;
-  const int N = G.N;
-  const size_t sb = 27ull * N * sizeof(R);
-  const int K = h->K;
-  const int nck = (int)(nsteps / K) + 1;
-  cudaStream_t s = h->stream;
-  const PopConsts<R>& k = kc<R>(h);
-  k_params_to_T<R><<<blocks(N), 256, 0, s>>>(theta, static_cast<R*>(h->T6), N);
-  ACK(cudaGetLastError(), "params");
-  R* ck = nullptr;
-  R* seg = nullptr;
-  ACK(cudaMallocAsync((void**)&ck, sb * nck, s), "checkpoint buffer");
-  ACK(cudaMallocAsync((void**)&seg, sb * (size_t)(K + 1), s), "segment buffer");
+cudaError_t forward(elbm_adjoint_ctx* h, const R* in, R* out, unsigned long long* fb) {
   const R* T6 = static_cast<const R*>(h->T6);
-  ACK(cudaMemsetAsync(h->fb, 0, sizeof(unsigned long long), s), "memset");
-  ACK(cudaMemsetAsync(h->part, 0, sizeof(double) * blocks(N) * (nobs + 1), s), "memset");
+  if constexpr (sizeof(R) == 8) {
+    if (h->fixed.fix.ok)
+      return launch_next(k_adj_forward_fixed, dim3(step_blocks(h->G.N, 64)), dim3(64), 0, h->stream, in, out, T6, h->G,
+                         h->fixed, fb);
+  }
+  constexpr int B = STEP_THREADS<R>;
+  return launch_next(k_adj_forward<R>, dim3(step_blocks(h->G.N, B)), dim3(B), 0, h->stream, in, out, T6, h->G, kc<R>(h), fb);
+}
+
+template <typename R>
+cudaError_t vjp(elbm_adjoint_ctx* h, const R* state, const R* gbar_next, R* gbar, const R* target, bool first) {
+  constexpr int B = STEP_THREADS<R>;
+  return launch_next(k_adj_vjp<R>, dim3(step_blocks(h->G.N, B)), dim3(B), 0, h->stream, state, gbar_next, gbar,
+                     static_cast<const R*>(h->T6), h->Tbar, target, h->G, kc<R>(h), first ? 1 : 0);
+}
+
+// Room for `bytes` of states in the handle's workspace.
+cudaError_t reserve(elbm_adjoint_ctx* h, size_t bytes) {
+  if (bytes <= h->state_bytes) return cudaSuccess;
+  cudaStreamSynchronize(h->stream);
+  cudaFree(h->states);
+  h->states = nullptr;
+  h->state_bytes = 0;
+  const cudaError_t e = cudaMalloc(&h->states, bytes);
+  if (e == cudaSuccess) h->state_bytes = bytes;
+  else cudaGetLastError();
+  return e;
+}
+
+template <typename R>
+elbm_status run_steps(elbm_adjoint_ctx* h, const R* theta, const R* phi0, int64_t nsteps, int nobs, const int64_t* obs,
+                      const R* targets, double* J, R* grad, int64_t* nfb) {
+  const int N = h->G.N;
+  const size_t S = 27ull * N, sb = S * sizeof(R);
+  cudaStream_t s = h->stream;
+  // Segments of K steps.  A forward run alone alternates between two states.  With a gradient, every
+  // state of the run is kept if they fit KEEP_BYTES (one segment); else checkpoints every
+  // h->K steps, and the states of one segment at a time.
+  int64_t K = nsteps, last = 0, t_last = 0;     // last segment, its first step
+  size_t ncheck = 1, nseg = 2;
+  const auto plan = [&](int64_t every) {
+    K = std::min<int64_t>(every, nsteps);
+    last = (nsteps - 1) / K;
+    t_last = last * K;
+    ncheck = (size_t)last + 1;
+    nseg = (size_t)K + 1;
+  };
+  if (grad != nullptr) plan((size_t)(nsteps + 2) <= KEEP_BYTES / sb ? nsteps : h->K);
+  cudaError_t e = reserve(h, (ncheck + nseg) * sb);
+  if (e == cudaErrorMemoryAllocation && grad != nullptr && K > h->K) {
+    plan(h->K);
+    e = reserve(h, (ncheck + nseg) * sb);
+  }
+  ACK(e, "state buffer");
+  R* const ck = static_cast<R*>(h->states);
+  R* const seg = ck + S * ncheck;
+  k_params_to_T<R><<<blocks(N), 256, 0, s>>>(theta, static_cast<R*>(h->T6), h->aux, N);
+  ACK(cudaGetLastError(), "params");
+  ACK(cudaMemsetAsync(h->fb, 0, 2 * sizeof(unsigned long long), s), "memset");
+  ACK(cudaMemsetAsync(h->part, 0, sizeof(double) * blocks(N) * nobs, s), "memset");
   auto obs_index = [&](int64_t t) {
     for (int o = 0; o < nobs; ++o)
       if (obs[o] == t) return o;
     return -1;
   };
-  // forward sweep: checkpoints every K steps, misfit at the observation steps
-  k_adj_init<R><<<blocks(N), 256, 0, s>>>(phi0, ck, N, k);
+  R* gin = static_cast<R*>(h->gbar[0]);    // Gbar^{t+1}
+  R* gout = static_cast<R*>(h->gbar[1]);   // Gbar^t
+  // forward sweep: checkpoints every K steps, all states of the last segment, misfit at the
+  // observation steps (at the last step it is also the seed Gbar^T_i = phi_T - target)
+  k_adj_init<R><<<blocks(N), 256, 0, s>>>(phi0, ck, N, kc<R>(h));
   ACK(cudaGetLastError(), "init");
-  R* cur = ck;          // state G^t
-  R* nxt = seg;         // scratch for the next state when not a checkpoint
+  const R* cur = ck;
   for (int64_t t = 0; t < nsteps; ++t) {
-    R* dst = ((t + 1) % K == 0) ? ck + 27ull * N * ((t + 1) / K) : (cur == seg ? seg + 27ull * N : seg);
-    k_adj_forward<R><<<blocks(N), 256, 0, s>>>(cur, dst, T6, G, k, h->fb);
-    ACK(cudaGetLastError(), "forward");
+    R* dst;
+    if (grad != nullptr && t >= t_last) dst = seg + S * (t + 1 - t_last);
+    else if (grad != nullptr && (t + 1) % K == 0) dst = ck + S * ((t + 1) / K);
+    else dst = cur == seg ? seg + S : seg;
+    ACK(forward<R>(h, cur, dst, h->fb), "forward");
     cur = dst;
     const int o = obs_index(t + 1);
     if (o >= 0) {
       k_adj_misfit<R><<<blocks(N), 256, 0, s>>>(cur, targets + (size_t)o * N, h->part + (size_t)o * blocks(N),
-                                               nullptr, N);
+                                               grad != nullptr && t + 1 == nsteps ? gin : nullptr, N);
       ACK(cudaGetLastError(), "misfit");
     }
   }
-  (void)nxt;
+  if (grad != nullptr) {
+    // reverse sweep, segment by segment from the end
+    if (obs_index(nsteps) < 0) ACK(cudaMemsetAsync(gin, 0, sb, s), "memset");
+    for (int64_t sgm = last; sgm >= 0; --sgm) {
+      const int64_t t0 = sgm * K;
+      const int64_t t1 = std::min<int64_t>(nsteps, t0 + K);
+      const auto state = [&](int64_t t) { return t == t0 ? ck + S * sgm : seg + S * (t - t0); };
+      if (sgm != last)
+        for (int64_t t = t0; t < t1 - 1; ++t) ACK(forward<R>(h, state(t), state(t + 1), h->fb + 1), "recompute");
+      for (int64_t t = t1 - 1; t >= t0; --t) {
+        const int o = obs_index(t);
+        const R* tgt = (o >= 0 && t > 0) ? targets + (size_t)o * N : nullptr;
+        ACK(vjp<R>(h, state(t), gin, gout, tgt, t == nsteps - 1), "vjp");
+        std::swap(gin, gout);
+      }
+    }
+    k_Tbar_to_params<R><<<blocks(N), 256, 0, s>>>(h->aux, h->Tbar, grad, N);
+    ACK(cudaGetLastError(), "chain rule");
+  }
   std::vector<double> part((size_t)blocks(N) * nobs);
   ACK(cudaMemcpyAsync(part.data(), h->part, part.size() * sizeof(double), cudaMemcpyDeviceToHost, s), "memcpy");
   unsigned long long fb = 0;
@@ -444,53 +606,20 @@ elbm_status run_t(elbm_adjoint_ctx* h, const R* theta, const R* phi0, int64_t ns
   for (double v : part) Jv += v;
   if (J) *J = Jv;
   if (nfb) *nfb = (int64_t)fb;
-  if (grad != nullptr) {
-    // reverse sweep, segment by segment from the end
-    R* gb0 = static_cast<R*>(h->gbar[0]);
-    R* gb1 = static_cast<R*>(h->gbar[1]);
-    ACK(cudaMemsetAsync(gb0, 0, sb, s), "memset");
-    ACK(cudaMemsetAsync(h->Tbar, 0, 6ull * N * sizeof(double), s), "memset");
-    const int o_last = obs_index(nsteps);
-    if (o_last >= 0) {
-      // seed: Gbar^T_i = phi_T - target (recompute G^T into seg[0..])
-      const int64_t t0 = (nsteps / K) * K;
-      R* st = ck + 27ull * N * (t0 / K);
-      for (int64_t t = t0; t < nsteps; ++t) {
-        R* dst = seg + 27ull * N * ((t - t0) % 2);
-        k_adj_forward<R><<<blocks(N), 256, 0, s>>>(st, dst, T6, G, k, h->fb);
-        st = dst;
-      }
-      k_adj_misfit<R><<<blocks(N), 256, 0, s>>>(st, targets + (size_t)o_last * N,
-                                               h->part + (size_t)nobs * blocks(N), gb0, N);
-      ACK(cudaGetLastError(), "seed");
-    }
-    R* gin = gb0;   // Gbar^{t+1}
-    R* gout = gb1;  // Gbar^t
-    for (int64_t sgm = (nsteps - 1) / K; sgm >= 0; --sgm) {
-      const int64_t t0 = sgm * K;
-      const int64_t t1 = std::min<int64_t>(nsteps, t0 + K);
-      // recompute G^{t0 .. t1-1} into seg[0 .. t1-t0-1]
-      ACK(cudaMemcpyAsync(seg, ck + 27ull * N * sgm, sb, cudaMemcpyDeviceToDevice, s), "memcpy");
-      for (int64_t t = t0; t < t1 - 1; ++t) {
-        k_adj_forward<R><<<blocks(N), 256, 0, s>>>(seg + 27ull * N * (t - t0), seg + 27ull * N * (t - t0 + 1), T6,
-                                                  G, k, h->fb);
-      }
-      ACK(cudaGetLastError(), "recompute");
-      for (int64_t t = t1 - 1; t >= t0; --t) {
-        const int o = obs_index(t);
-        const R* tgt = (o >= 0 && t > 0) ? targets + (size_t)o * N : nullptr;
-        k_adj_vjp<R><<<blocks(N), 256, 0, s>>>(seg + 27ull * N * (t - t0), gin, gout, T6, h->Tbar, tgt, G, k);
-        std::swap(gin, gout);
-      }
-      ACK(cudaGetLastError(), "vjp");
-    }
-    k_Tbar_to_params<R><<<blocks(N), 256, 0, s>>>(theta, h->Tbar, grad, N);
-    ACK(cudaGetLastError(), "chain rule");
-  }
-  ACK(cudaFreeAsync(ck, s), "free");
-  ACK(cudaFreeAsync(seg, s), "free");
-  ACK(cudaStreamSynchronize(s), "sync");
   return ELBM_OK;
+}
+
+template <typename R>
+elbm_status run_t(elbm_adjoint_ctx* h, const R* theta, const R* phi0, int64_t nsteps, int nobs, const int64_t* obs,
+                  const R* targets, double* J, R* grad, int64_t* nfb) {
+  const elbm_status st = run_steps<R>(h, theta, phi0, nsteps, nobs, obs, targets, J, grad, nfb);
+  if (h->state_bytes > KEEP_BYTES) {
+    cudaStreamSynchronize(h->stream);
+    cudaFree(h->states);
+    h->states = nullptr;
+    h->state_bytes = 0;
+  }
+  return st;
 }
 
 }  // namespace
@@ -514,8 +643,9 @@ elbm_status elbm_adjoint_create(const int64_t dims[3], elbm_precision prec, void
   cudaError_t e = cudaMalloc(&h->T6, 6 * (size_t)N * rs);
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->Tbar, 6 * (size_t)N * sizeof(double));
   for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = cudaMalloc(&h->gbar[b], 27 * (size_t)N * rs);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->fb, sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->part, sizeof(double) * blocks((int)N) * 17);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->aux, 12 * (size_t)N * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->fb, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->part, sizeof(double) * blocks((int)N) * 16);
   if (e != cudaSuccess) {
     elbm_adjoint_destroy(h);
     return e == cudaErrorMemoryAllocation ? ELBM_ERR_OOM : ELBM_ERR_CUDA;
@@ -532,6 +662,8 @@ void elbm_adjoint_destroy(elbm_adjoint_handle h) {
   cudaFree(h->Tbar);
   cudaFree(h->gbar[0]);
   cudaFree(h->gbar[1]);
+  cudaFree(h->aux);
+  cudaFree(h->states);
   cudaFree(h->fb);
   cudaFree(h->part);
   delete h;
@@ -570,19 +702,16 @@ static elbm_status step_t(elbm_adjoint_ctx* h, const R* theta, const R* g, const
                           R* grad) {
   const int N = h->G.N;
   cudaStream_t s = h->stream;
-  k_params_to_T<R><<<blocks(N), 256, 0, s>>>(theta, static_cast<R*>(h->T6), N);
+  k_params_to_T<R><<<blocks(N), 256, 0, s>>>(theta, static_cast<R*>(h->T6), h->aux, N);
   ACK(cudaGetLastError(), "params");
-  if (g_next) {
-    k_adj_forward<R><<<blocks(N), 256, 0, s>>>(g, g_next, static_cast<const R*>(h->T6), h->G, kc<R>(h), h->fb);
-    ACK(cudaGetLastError(), "forward");
-  }
+  // (also keeps the step kernels, which may start before the kernel in front of them ends, from
+  // meeting an unfinished T6)
+  ACK(cudaMemsetAsync(h->fb, 0, 2 * sizeof(unsigned long long), s), "memset");
+  if (g_next) ACK(forward<R>(h, g, g_next, h->fb), "forward");
   if (gbar) {
-    ACK(cudaMemsetAsync(h->Tbar, 0, 6ull * N * sizeof(double), s), "memset");
-    k_adj_vjp<R><<<blocks(N), 256, 0, s>>>(g, gbar_next, gbar, static_cast<const R*>(h->T6), h->Tbar, nullptr, h->G,
-                                          kc<R>(h));
-    ACK(cudaGetLastError(), "vjp");
+    ACK(vjp<R>(h, g, gbar_next, gbar, nullptr, true), "vjp");
     if (grad) {
-      k_Tbar_to_params<R><<<blocks(N), 256, 0, s>>>(theta, h->Tbar, grad, N);
+      k_Tbar_to_params<R><<<blocks(N), 256, 0, s>>>(h->aux, h->Tbar, grad, N);
       ACK(cudaGetLastError(), "chain rule");
     }
   }
