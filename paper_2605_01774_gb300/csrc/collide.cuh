@@ -130,7 +130,7 @@ __device__ __forceinline__ void node_tables(PopConsts<R>& kn, R ux, R uy, R uz) 
   for (int i = 0; i < Q; ++i) {
     const R cu = R(cx_of(i)) * ux + R(cy_of(i)) * uy + R(cz_of(i)) * uz;
     if constexpr (sizeof(R) == 4) {
-      eq_tables_f32(fmaf(3.0f, cu, __fmul_rn(-1.5f, uu)), __fmul_rn(__fmul_rn(4.5f, cu), cu), float(w_of(i)), kn.E[i],
+      eq_tables_f32<false>(fmaf(3.0f, cu, __fmul_rn(-1.5f, uu)), __fmul_rn(__fmul_rn(4.5f, cu), cu), float(w_of(i)), kn.E[i],
                     kn.K3[i], kn.L[i], kn.M[i]);
     } else {
       const R P = R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * uu;
@@ -146,32 +146,41 @@ __device__ __forceinline__ void node_tables(PopConsts<R>& kn, R ux, R uy, R uz) 
   kn.uz = uz;
 }
 
-// VEL = 0: u = 0 exactly (kappa = 0); VEL = 1: uniform u from PopConsts; VEL = 2: the
-// node's own velocity un[3] (tables rebuilt per node; lambda = 1 where that u is exactly 0).
-// ROOT: lambda from the exact entropy root (k.root); a separate instantiation, so the FP64
-// Newton arrays cost the closed-form kernels no registers.
-// Returns true if the positivity fallback was taken; phi_out receives the node's phi,
-// which the collision conserves exactly.
-template <typename R, int VEL, bool ROOT = false>
-__device__ __forceinline__ bool collide_node(R (&g)[Q], const Sym6<R>& T, const PopConsts<R>& k,
-                                             bool fallback, R& phi_out, const R* un = nullptr) {
-  if constexpr (VEL == 2) {
-    PopConsts<R> kn = k;
-    if (un[0] == R(0) && un[1] == R(0) && un[2] == R(0)) {
-      node_tables(kn, R(0), R(0), R(0));
-      return collide_node<R, 0>(g, T, kn, fallback, phi_out);
-    }
-    node_tables(kn, un[0], un[1], un[2]);
-    return collide_node<R, 1, ROOT>(g, T, kn, fallback, phi_out);
+// The tables of a collision: those of PopConsts, or (FP32 velocity fields) of the node's velocity,
+// each population's computed where the stabilizer's sums use it.  Computed ahead, the 108 values
+// do not fit the registers.
+template <typename R>
+struct UniformTables {
+  static constexpr bool LAZY = false;
+  const PopConsts<R>& k;
+  __device__ __forceinline__ void at(int i, R& E, R& K3, R& L, R& M) const {
+    E = k.E[i];
+    K3 = k.K3[i];
+    L = k.L[i];
+    M = k.M[i];
   }
+};
+template <bool SERIES>   // series_range holds
+struct NodeTables {
+  static constexpr bool LAZY = true;
+  float ux, uy, uz, odd;   // odd: -1.5 u.u
+  __device__ __forceinline__ void at(int i, float& E, float& K3, float& L, float& M) const {
+    const float cu = float(cx_of(i)) * ux + float(cy_of(i)) * uy + float(cz_of(i)) * uz;
+    eq_tables_f32<SERIES>(fmaf(3.0f, cu, odd), __fmul_rn(__fmul_rn(4.5f, cu), cu), float(w_of(i)), E, K3, L, M);
+  }
+};
+
+template <typename R, int VEL, bool ROOT, typename Tables>
+__device__ __forceinline__ bool collide_with(R (&g)[Q], const Sym6<R>& T, const PopConsts<R>& k, const Tables& tables,
+                                             R ux, R uy, R uz, bool fallback, R& phi_out) {
   R phi, mx, my, mz;
   moments(g, phi, mx, my, mz);
   phi_out = phi;
   R jx = mx, jy = my, jz = mz;
   if (VEL == 1) {
-    jx = mx - phi * k.ux;
-    jy = my - phi * k.uy;
-    jz = mz - phi * k.uz;
+    jx = mx - phi * ux;
+    jy = my - phi * uy;
+    jz = mz - phi * uz;
   }
   R tx, ty, tz;
   sym_mul(T, jx, jy, jz, tx, ty, tz);
@@ -187,20 +196,23 @@ __device__ __forceinline__ bool collide_node(R (&g)[Q], const Sym6<R>& T, const 
     // underflow in FP32 and the guard reads sum (dh/phi)^2 M > theta^2.
     R kappa = R(0);
     const R tiny = sizeof(R) == 4 ? R(1e-30) : R(1e-300);
-    if (phi > tiny) {
+    R E[Q];
+    if (Tables::LAZY || phi > tiny) {
       // FP32: reciprocal-based quotients (2 ulp); inv only normalises the H-products
-      const R inv = sizeof(R) == 4 ? R(__fdividef(1.0f, float(phi))) : R(1) / phi;
+      const R inv = phi > tiny ? (sizeof(R) == 4 ? R(__fdividef(1.0f, float(phi))) : R(1) / phi) : R(0);
       const Dots<R> cj(jx * inv, jy * inv, jz * inv);
       const Dots<R> ca(ax * inv, ay * inv, az * inv);
       R num = R(0), den = R(0);
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        R dh = g[i] * inv - k.E[i];
+        R K3, L, M;
+        tables.at(i, E[i], K3, L, M);
+        R dh = g[i] * inv - E[i];
         dh = dh - R(3.0 * w_of(i)) * cj.d[i];
-        num += dh * (k.K3[i] * ca.d[i] + k.L[i]);
-        den += dh * (dh * k.M[i]);
+        num += dh * (K3 * ca.d[i] + L);
+        den += dh * (dh * M);
       }
-      if (den > k.theta2) {
+      if (den > k.theta2 && (!Tables::LAZY || phi > tiny)) {
         kappa = sizeof(R) == 4 ? R(__fdividef(float(num), float(den))) : num / den;
         if constexpr (ROOT) {
           double geq[Q], dsp[Q], dhd[Q], L[Q];
@@ -219,7 +231,7 @@ __device__ __forceinline__ bool collide_node(R (&g)[Q], const Sym6<R>& T, const 
     const R psi = (R(1) + kappa) * phi;
     const Dots<R> cb(ax + kappa * jx, ay + kappa * jy, az + kappa * jz);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) gs[i] = psi * k.E[i] - kappa * g[i] + R(3.0 * w_of(i)) * cb.d[i];
+    for (int i = 0; i < Q; ++i) gs[i] = psi * (Tables::LAZY ? E[i] : k.E[i]) - kappa * g[i] + R(3.0 * w_of(i)) * cb.d[i];
   }
   bool took = false;
   if (fallback) {
@@ -281,6 +293,35 @@ __device__ __forceinline__ bool collide_node(R (&g)[Q], const Sym6<R>& T, const 
 #pragma unroll
   for (int i = 0; i < Q; ++i) g[i] = gs[i];
   return took;
+}
+
+// VEL = 0: u = 0 exactly (kappa = 0); VEL = 1: uniform u from PopConsts; VEL = 2: the
+// node's own velocity un[3] (tables rebuilt per node; lambda = 1 where that u is exactly 0).
+// ROOT: lambda from the exact entropy root (k.root); a separate instantiation, so the FP64
+// Newton arrays cost the closed-form kernels no registers.
+// Returns true if the positivity fallback was taken; phi_out receives the node's phi,
+// which the collision conserves exactly.
+template <typename R, int VEL, bool ROOT = false>
+__device__ __forceinline__ bool collide_node(R (&g)[Q], const Sym6<R>& T, const PopConsts<R>& k,
+                                             bool fallback, R& phi_out, const R* un = nullptr) {
+  if constexpr (VEL == 2) {
+    if (un[0] == R(0) && un[1] == R(0) && un[2] == R(0))
+      return collide_with<R, 0, false>(g, T, k, UniformTables<R>{k}, R(0), R(0), R(0), fallback, phi_out);
+    if constexpr (sizeof(R) == 4 && !ROOT) {
+      const float uu = un[0] * un[0] + un[1] * un[1] + un[2] * un[2], odd = __fmul_rn(-1.5f, uu);
+      if (series_range(fabsf(un[0]) + fabsf(un[1]) + fabsf(un[2]), uu))
+        return collide_with<R, 1, false>(g, T, k, NodeTables<true>{un[0], un[1], un[2], odd}, un[0], un[1], un[2],
+                                         fallback, phi_out);
+      return collide_with<R, 1, false>(g, T, k, NodeTables<false>{un[0], un[1], un[2], odd}, un[0], un[1], un[2],
+                                       fallback, phi_out);
+    } else {
+      PopConsts<R> kn = k;
+      node_tables(kn, un[0], un[1], un[2]);
+      return collide_with<R, 1, ROOT>(g, T, kn, UniformTables<R>{kn}, un[0], un[1], un[2], fallback, phi_out);
+    }
+  } else {
+    return collide_with<R, VEL, ROOT>(g, T, k, UniformTables<R>{k}, k.ux, k.uy, k.uz, fallback, phi_out);
+  }
 }
 
 }  // namespace elbm

@@ -59,7 +59,7 @@ __device__ __forceinline__ void node_tables2(Consts2<R>& k, R ux, R uy) {
   for (int i = 0; i < Q2; ++i) {
     const R cu = R(cx2(i)) * ux + R(cy2(i)) * uy;
     if constexpr (sizeof(R) == 4) {
-      elbm::eq_tables_f32(fmaf(3.0f, cu, __fmul_rn(-1.5f, uu)), __fmul_rn(__fmul_rn(4.5f, cu), cu), float(w2(i)),
+      elbm::eq_tables_f32<false>(fmaf(3.0f, cu, __fmul_rn(-1.5f, uu)), __fmul_rn(__fmul_rn(4.5f, cu), cu), float(w2(i)),
                           k.E[i], k.K3[i], k.L[i], k.M[i]);
     } else {
       const R P = R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * uu;
