@@ -8,63 +8,49 @@
 
 namespace elbm {
 
-// Resident blocks per SM requested from the register allocator (256 threads each).
+// Nodes are dealt out in a row, 64 to a block: no lane is lost to the ends of rows, small lattices
+// reach all SMs, and the node's coordinates (two divisions) are worked out while the launch waits for
+// the one before.  Against blocks of 256 that each took pieces of rows (whole passes: steps, start
+// and read-outs): 24^3 FP32 plume 171 -> 127 us, 48 x 40 x 32 FP32 at rest 364 -> 352 us (100 steps),
+// 121 x 75 x 50 FP32 porous 1043 -> 962 us, 190 x 200 x 180 FP32 porous 3.59 -> 3.16 ms, 200 x 200 x
+// 190 FP16 plume 3.04 -> 2.70 ms.  With the divisions after the wait 24^3 137, at rest 422 us; blocks
+// of 128 then 141 and 396 us.
+constexpr int THREADS = 64;
+
+// Resident warps per SM requested from the register allocator, in units of 8.
 #ifndef ELBM_STEP_MINB
 #define ELBM_STEP_MINB 3
 #endif
-template <typename Elem>
-__host__ __device__ constexpr int step_min_blocks() {
-  return std::is_same<Elem, double>::value ? 1 : ELBM_STEP_MINB;
-}
-
-// Threads per block and blocks per SM of the fixed-point FP64 kernel: 34 KB of shared memory per
-// 64 nodes (fixed.cuh) lets 6 blocks stand on an SM at 168 registers.  Measured on the 96 x 80 x 72
-// plume, 20 steps and their read-outs: 4 blocks 4.09, 6 blocks 3.69 ms; all loops unrolled, no
-// shared memory, 2 to 4 blocks of 128 3.97 to 4.24 ms (waiting for instructions); FP64 arithmetic
-// 10.7 ms.
-#ifndef ELBM_FIXED_THREADS
-#define ELBM_FIXED_THREADS 64
-#endif
+// FP64 in fixed point: 34 KB of shared memory per 64 nodes (fixed.cuh) lets 6 blocks stand on an SM
+// at 168 registers.  Measured on the 96 x 80 x 72 plume, 20 steps and their read-outs: 4 blocks 4.09,
+// 6 blocks 3.69 ms; all loops unrolled, no shared memory, 2 to 4 blocks of 128 3.97 to 4.24 ms
+// (waiting for instructions); FP64 arithmetic 10.7 ms.
 #ifndef ELBM_FIXED_MINB
 #define ELBM_FIXED_MINB 6
 #endif
 template <typename Elem, int MODE>
-__host__ __device__ constexpr int step_threads() {
-  return MODE == FIXED ? ELBM_FIXED_THREADS : 256;
-}
-template <typename Elem, int MODE>
 __host__ __device__ constexpr int step_blocks() {
-  return MODE == FIXED ? ELBM_FIXED_MINB : step_min_blocks<Elem>();
+  return MODE == FIXED ? ELBM_FIXED_MINB : (std::is_same<Elem, double>::value ? 1 : ELBM_STEP_MINB) * (256 / THREADS);
 }
 
 template <int MODE>
-using Kept = typename std::conditional<MODE == FIXED, InShared<ELBM_FIXED_THREADS>, KeepNone>::type;
+using Kept = typename std::conditional<MODE == FIXED, InShared<THREADS>, KeepNone>::type;
 
 template <typename Elem, int VEL, int MODE>
-__global__ void __launch_bounds__(step_threads<Elem, MODE>(), step_blocks<Elem, MODE>())
+__global__ void __launch_bounds__(THREADS, step_blocks<Elem, MODE>())
 k_step(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G,
        const typename Storage<Elem>::real* __restrict__ T6,
        const float* __restrict__ src, const float* __restrict__ u3, int fallback,
        unsigned long long* __restrict__ counters, const PopConsts<typename Storage<Elem>::real> k,
        const __grid_constant__ StepConsts<MODE> c) {
   using R = typename Storage<Elem>::real;
+  const unsigned m = blockIdx.x * (unsigned)THREADS + threadIdx.x, row = m / (unsigned)G.nx;
+  const int x = (int)(m - row * (unsigned)G.nx), y = (int)(row % (unsigned)G.ny), z = (int)(row / (unsigned)G.ny);
+  __shared__ int64_t kept[MODE == FIXED ? KEPT * THREADS : 1];
   wait_for_previous();
-  int x, y, z;
-  if constexpr (MODE == FIXED) {
-    // long collisions: nodes in a row, so that no lane is lost to the ends of short rows
-    const unsigned m = blockIdx.x * (unsigned)step_threads<Elem, MODE>() + threadIdx.x, row = m / (unsigned)G.nx;
-    x = (int)(m - row * (unsigned)G.nx);
-    y = (int)(row % (unsigned)G.ny);
-    z = (int)(row / (unsigned)G.ny);
-  } else {
-    x = blockIdx.x * blockDim.x + threadIdx.x;
-    y = blockIdx.y * blockDim.y + threadIdx.y;
-    z = blockIdx.z;
-  }
-  __shared__ int64_t kept[MODE == FIXED ? KEPT * step_threads<Elem, MODE>() : 1];
   bool took = false, proj = false;
-  if (x < G.nx && y < G.ny && z < G.nz) {
-    const int n = x + G.nx * (y + G.ny * z);
+  if (z < G.nz) {
+    const int n = (int)m;
     R g[Q];
     pull_node<Elem, R>(g, in, G, x, y, z, k);
     // merged Strang half-steps of consecutive steps (Section 3.3)
@@ -83,10 +69,10 @@ k_step(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G
   }
   // one counter update per block
   const int cnt = __syncthreads_count(took);
-  if (cnt != 0 && threadIdx.x == 0 && threadIdx.y == 0) atomicAdd(counters, (unsigned long long)cnt);
+  if (cnt != 0 && threadIdx.x == 0) atomicAdd(counters, (unsigned long long)cnt);
   if constexpr (Storage<Elem>::dev) {
     const int p = __syncthreads_count(proj);
-    if (p != 0 && threadIdx.x == 0 && threadIdx.y == 0) atomicAdd(counters + 3, (unsigned long long)p);
+    if (p != 0 && threadIdx.x == 0) atomicAdd(counters + 3, (unsigned long long)p);
   }
 }
 
@@ -95,14 +81,10 @@ static cudaError_t launch_t(const StepLaunch& L, cudaStream_t s) {
   using R = typename Storage<Elem>::real;
   Field<Elem> in{static_cast<const Elem*>(L.pin), L.sin};
   Grid G{L.nx, L.ny, L.nz, L.N, L.dirichlet};
-  dim3 b = row_block(L.nx), g = row_grid(b, L.nx, L.ny, L.nz);
-  if constexpr (MODE == FIXED) {
-    b = dim3(step_threads<Elem, MODE>());
-    g = dim3((unsigned)((L.N + b.x - 1) / b.x));
-  }
   const PopConsts<R>& k = *reinterpret_cast<const PopConsts<R>*>(std::is_same<R, double>::value ? (const void*)L.kd
                                                                                                : (const void*)L.kf);
-  return launch_next(k_step<Elem, VEL, MODE>, g, b, 0, s, in, static_cast<Elem*>(L.pout), L.sout, G,
+  const dim3 blocks((unsigned)((L.N + THREADS - 1) / THREADS));
+  return launch_next(k_step<Elem, VEL, MODE>, blocks, dim3(THREADS), 0, s, in, static_cast<Elem*>(L.pout), L.sout, G,
                      static_cast<const R*>(L.T6), L.src, L.u3, L.fallback, L.counters, k, step_consts<MODE>(L));
 }
 
