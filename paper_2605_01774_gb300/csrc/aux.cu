@@ -8,6 +8,12 @@ namespace elbm {
 
 namespace {
 
+// Threads per block of the state transfers, nodes dealt out in a row.
+#ifndef ELBM_IO_THREADS
+#define ELBM_IO_THREADS 64
+#endif
+constexpr int THREADS = ELBM_IO_THREADS;
+
 template <typename T>
 __device__ __forceinline__ double ld_in(const void* p, size_t idx) {
   return (double)static_cast<const T*>(p)[idx];
@@ -30,16 +36,15 @@ __device__ __forceinline__ R shape_at(const float* __restrict__ u3, size_t N, in
 // (anti-bounce-back inverted: the stored outgoing population of a wall node only
 // feeds the entering opposite one).
 template <typename Elem, typename Tin, int FROM_PHI>
-__global__ void __launch_bounds__(256, 2)   // 128^3 FP64 with source 447 us, unbounded 530; 256^3 FP32 402, with 3 blocks 462
+__global__ void __launch_bounds__(THREADS, 512 / THREADS)   // 128^3 FP64 with source 447 us, unbounded 530; 256^3 FP32 402, with 3 blocks 462
 k_write(Elem* __restrict__ pops, float* __restrict__ scale, Grid G, const void* __restrict__ in,
         const float* __restrict__ src, const float* __restrict__ u3,
         const PopConsts<typename Storage<Elem>::real> k) {
   using R = typename Storage<Elem>::real;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = blockIdx.z;
-  if (x >= G.nx || y >= G.ny) return;
-  const int n = x + G.nx * (y + G.ny * z);
+  const unsigned m = blockIdx.x * (unsigned)THREADS + threadIdx.x, row = m / (unsigned)G.nx;
+  const int x = (int)(m - row * (unsigned)G.nx), y = (int)(row % (unsigned)G.ny), z = (int)(row / (unsigned)G.ny);
+  if (z >= G.nz) return;
+  const int n = (int)m;
   // All 27 destinations are loaded at once (wrapped, as if periodic), then the uniform cases, then
   // the faces: with the cases inside the loop every load waited for the one before it (256^3 FP32
   // 0.50 -> 0.40 ms, FP16 deviations 0.56 -> 0.39 ms).
@@ -82,17 +87,16 @@ k_write(Elem* __restrict__ pops, float* __restrict__ scale, Grid G, const void* 
 
 // ----------------------------------------------------------------- read state
 template <typename Elem, typename Tout, int WHAT>
-__global__ void __launch_bounds__(256, 3)   // FP16 phi of 256^3: 281 us, with up to 2 or 4 blocks 367 and 304
+__global__ void __launch_bounds__(THREADS, 768 / THREADS)   // FP16 phi of 256^3: 281 us, with up to 2 or 4 blocks 367 and 304
 k_read(Field<Elem> f, Grid G, Tout* __restrict__ out, Tout* __restrict__ qout,
        const typename Storage<Elem>::real* __restrict__ T6,
        const float* __restrict__ src, const float* __restrict__ u3,
        const PopConsts<typename Storage<Elem>::real> k) {
   using R = typename Storage<Elem>::real;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = blockIdx.z;
-  if (x >= G.nx || y >= G.ny) return;
-  const int n = x + G.nx * (y + G.ny * z);
+  const unsigned m = blockIdx.x * (unsigned)THREADS + threadIdx.x, row = m / (unsigned)G.nx;
+  const int x = (int)(m - row * (unsigned)G.nx), y = (int)(row % (unsigned)G.ny), z = (int)(row / (unsigned)G.ny);
+  if (z >= G.nz) return;
+  const int n = (int)m;
   R g[Q];
   pull_node<Elem, R>(g, f, G, x, y, z, k);
   if (src != nullptr) {
@@ -207,7 +211,7 @@ const PopConsts<typename Storage<Elem>::real>& consts_of(const StateIO& S) {
 template <typename Elem>
 cudaError_t write_t(const StateIO& S, const void* in, int in_f32, int from_phi, cudaStream_t s) {
   Grid G{S.nx, S.ny, S.nz, S.N, S.dirichlet};
-  dim3 b = row_block(S.nx), g = row_grid(b, S.nx, S.ny, S.nz);
+  const dim3 b(THREADS), g((unsigned)((S.N + THREADS - 1) / THREADS));
   Elem* p = static_cast<Elem*>(S.pops);
   const auto& k = consts_of<Elem>(S);
   if (in_f32) {
@@ -223,7 +227,7 @@ cudaError_t write_t(const StateIO& S, const void* in, int in_f32, int from_phi, 
 template <typename Elem>
 cudaError_t read_t(const StateIO& S, void* out, void* q, int out_f32, int what, cudaStream_t s) {
   Grid G{S.nx, S.ny, S.nz, S.N, S.dirichlet};
-  dim3 b = row_block(S.nx), g = row_grid(b, S.nx, S.ny, S.nz);
+  const dim3 b(THREADS), g((unsigned)((S.N + THREADS - 1) / THREADS));
   using R = typename Storage<Elem>::real;
   const auto& k = consts_of<Elem>(S);
   Field<Elem> f = field_of<Elem>(S);
