@@ -404,10 +404,9 @@ static elbm_status write_state(elbm_handle h, const void* in, elbm_dtype dt, int
   elbm_status s = to_device(h, in, bytes, &dev, &tmp);
   if (s != ELBM_OK) return s;
   StateIO S = state_io(h);
+  S.reset = h->d_counters;
   CK(launch_write_state(S, dev, dt == ELBM_DTYPE_F32, from_phi, h->stream), "write state");
   if (tmp) CK(cudaFreeAsync(tmp, h->stream), "cudaFreeAsync");
-  CK(cudaMemsetAsync(h->d_counters, 0, sizeof(unsigned long long), h->stream), "memset");
-  CK(cudaMemsetAsync(h->d_counters + 3, 0, sizeof(unsigned long long), h->stream), "memset");
   h->step = 0;
   h->initialized = true;
   return ELBM_OK;

@@ -14,6 +14,8 @@ namespace {
 #endif
 constexpr int THREADS = ELBM_IO_THREADS;
 
+// The transfers are launched like steps (launch.cuh); what the caller's kernels write is read with plain
+// loads, which do not move over the wait.
 template <typename T>
 __device__ __forceinline__ double ld_in(const void* p, size_t idx) {
   return (double)static_cast<const T*>(p)[idx];
@@ -21,7 +23,7 @@ __device__ __forceinline__ double ld_in(const void* p, size_t idx) {
 
 // E_i(u) at node d of a velocity field.
 template <typename R>
-__device__ __forceinline__ R shape_at(const float* __restrict__ u3, size_t N, int d, int i) {
+__device__ __forceinline__ R shape_at(const float* u3, size_t N, int d, int i) {
   const R ux = u3[d], uy = u3[N + d], uz = u3[2 * N + d];
   const R cu = R(cx_of(i)) * ux + R(cy_of(i)) * uy + R(cz_of(i)) * uz;
   return R(w_of(i)) * (R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * (ux * ux + uy * uy + uz * uz));
@@ -37,12 +39,13 @@ __device__ __forceinline__ R shape_at(const float* __restrict__ u3, size_t N, in
 // feeds the entering opposite one).
 template <typename Elem, typename Tin, int FROM_PHI>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS)   // 128^3 FP64 with source 447 us, unbounded 530; 256^3 FP32 402, with 3 blocks 462
-k_write(Elem* __restrict__ pops, float* __restrict__ scale, Grid G, const void* __restrict__ in,
-        const float* __restrict__ src, const float* __restrict__ u3,
-        const PopConsts<typename Storage<Elem>::real> k) {
+k_write(Elem* __restrict__ pops, float* __restrict__ scale, Grid G, const void* in, const float* src, const float* u3,
+        unsigned long long* reset, const PopConsts<typename Storage<Elem>::real> k) {
   using R = typename Storage<Elem>::real;
   const unsigned m = blockIdx.x * (unsigned)THREADS + threadIdx.x, row = m / (unsigned)G.nx;
   const int x = (int)(m - row * (unsigned)G.nx), y = (int)(row % (unsigned)G.ny), z = (int)(row / (unsigned)G.ny);
+  wait_for_previous();
+  if (m == 0 && reset != nullptr) reset[0] = reset[3] = 0ull;
   if (z >= G.nz) return;
   const int n = (int)m;
   // All 27 destinations are loaded at once (wrapped, as if periodic), then the uniform cases, then
@@ -89,12 +92,12 @@ k_write(Elem* __restrict__ pops, float* __restrict__ scale, Grid G, const void* 
 template <typename Elem, typename Tout, int WHAT>
 __global__ void __launch_bounds__(THREADS, 768 / THREADS)   // FP16 phi of 256^3: 281 us, with up to 2 or 4 blocks 367 and 304
 k_read(Field<Elem> f, Grid G, Tout* __restrict__ out, Tout* __restrict__ qout,
-       const typename Storage<Elem>::real* __restrict__ T6,
-       const float* __restrict__ src, const float* __restrict__ u3,
+       const typename Storage<Elem>::real* __restrict__ T6, const float* src, const float* u3,
        const PopConsts<typename Storage<Elem>::real> k) {
   using R = typename Storage<Elem>::real;
   const unsigned m = blockIdx.x * (unsigned)THREADS + threadIdx.x, row = m / (unsigned)G.nx;
   const int x = (int)(m - row * (unsigned)G.nx), y = (int)(row % (unsigned)G.ny), z = (int)(row / (unsigned)G.ny);
+  wait_for_previous();
   if (z >= G.nz) return;
   const int n = (int)m;
   R g[Q];
@@ -214,14 +217,9 @@ cudaError_t write_t(const StateIO& S, const void* in, int in_f32, int from_phi, 
   const dim3 b(THREADS), g((unsigned)((S.N + THREADS - 1) / THREADS));
   Elem* p = static_cast<Elem*>(S.pops);
   const auto& k = consts_of<Elem>(S);
-  if (in_f32) {
-    if (from_phi) k_write<Elem, float, 1><<<g, b, 0, s>>>(p, S.scale, G, in, S.src, S.u3, k);
-    else k_write<Elem, float, 0><<<g, b, 0, s>>>(p, S.scale, G, in, S.src, S.u3, k);
-  } else {
-    if (from_phi) k_write<Elem, double, 1><<<g, b, 0, s>>>(p, S.scale, G, in, S.src, S.u3, k);
-    else k_write<Elem, double, 0><<<g, b, 0, s>>>(p, S.scale, G, in, S.src, S.u3, k);
-  }
-  return cudaGetLastError();
+  auto kernel = in_f32 ? (from_phi ? k_write<Elem, float, 1> : k_write<Elem, float, 0>)
+                       : (from_phi ? k_write<Elem, double, 1> : k_write<Elem, double, 0>);
+  return launch_next(kernel, g, b, 0, s, p, S.scale, G, in, S.src, S.u3, S.reset, k);
 }
 
 template <typename Elem>
@@ -232,14 +230,11 @@ cudaError_t read_t(const StateIO& S, void* out, void* q, int out_f32, int what, 
   const auto& k = consts_of<Elem>(S);
   Field<Elem> f = field_of<Elem>(S);
   const R* T6 = static_cast<const R*>(S.T6);
-  if (out_f32) {
-    if (what == 0) k_read<Elem, float, 0><<<g, b, 0, s>>>(f, G, (float*)out, (float*)q, T6, S.src, S.u3, k);
-    else k_read<Elem, float, 1><<<g, b, 0, s>>>(f, G, (float*)out, (float*)q, T6, S.src, S.u3, k);
-  } else {
-    if (what == 0) k_read<Elem, double, 0><<<g, b, 0, s>>>(f, G, (double*)out, (double*)q, T6, S.src, S.u3, k);
-    else k_read<Elem, double, 1><<<g, b, 0, s>>>(f, G, (double*)out, (double*)q, T6, S.src, S.u3, k);
-  }
-  return cudaGetLastError();
+  if (out_f32)
+    return launch_next(what == 0 ? k_read<Elem, float, 0> : k_read<Elem, float, 1>, g, b, 0, s, f, G, (float*)out,
+                       (float*)q, T6, S.src, S.u3, k);
+  return launch_next(what == 0 ? k_read<Elem, double, 0> : k_read<Elem, double, 1>, g, b, 0, s, f, G, (double*)out,
+                     (double*)q, T6, S.src, S.u3, k);
 }
 
 template <typename Elem>

@@ -56,6 +56,7 @@ struct StateIO {
   const float* src;
   const PopConsts<double>* kd;
   const PopConsts<float>* kf;
+  unsigned long long* reset = nullptr;   // write: counters [0] and [3] of this array are set to 0
 };
 cudaError_t launch_write_state(const StateIO& S, const void* in, int in_f32, int from_phi, cudaStream_t s);
 // what: 0 = populations [27][N]; 1 = phi [N] and optional q [3][N]
