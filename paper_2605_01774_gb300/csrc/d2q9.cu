@@ -166,7 +166,8 @@ int row_pieces(int nx, int ny) {
 template <typename R, int VEL, bool ROWS>
 __global__ void __launch_bounds__(THREADS2)
 k_step2(const R* in, R* out, Grid2 G, const R* __restrict__ T3,
-        const float* __restrict__ u2, int fallback, unsigned long long* __restrict__ counters, const Consts2<R> k) {
+        const float* __restrict__ u2, const R* __restrict__ tab, int fallback,
+        unsigned long long* __restrict__ counters, const Consts2<R> k) {
   int x, y;
   if constexpr (ROWS) {
     x = (int)(blockIdx.x * (unsigned)THREADS2 + threadIdx.x);
@@ -193,7 +194,20 @@ k_step2(const R* in, R* out, Grid2 G, const R* __restrict__ T3,
       tyy = __ldg(T3 + 2 * G.N + n);
     }
     bool t;
-    if constexpr (VEL == 2) {
+    if constexpr (VEL == 3) {
+      Consts2<R> kn = k;
+      kn.ux = R(__ldg(u2 + n));
+      kn.uy = R(__ldg(u2 + G.N + n));
+#pragma unroll
+      for (int i = 0; i < Q2; ++i) {
+        kn.E[i] = __ldg(tab + (size_t)i * G.N + n);
+        kn.K3[i] = __ldg(tab + (size_t)(Q2 + i) * G.N + n);
+        kn.L[i] = __ldg(tab + (size_t)(2 * Q2 + i) * G.N + n);
+        kn.M[i] = __ldg(tab + (size_t)(3 * Q2 + i) * G.N + n);
+      }
+      t = kn.ux == R(0) && kn.uy == R(0) ? collide2<R, 0>(g, txx, txy, tyy, kn, fallback != 0)
+                                         : collide2<R, 1>(g, txx, txy, tyy, kn, fallback != 0);
+    } else if constexpr (VEL == 2) {
       const R ux = R(__ldg(u2 + n)), uy = R(__ldg(u2 + G.N + n));
       Consts2<R> kn = k;
       if (ux == R(0) && uy == R(0)) {
@@ -322,6 +336,26 @@ __global__ void k_velocity_check2(const float* __restrict__ u2, size_t N, unsign
   }
 }
 
+// The tables E, K3, L, M of a velocity field's nodes, [4][9][N], for FP64 handles: the field is fixed
+// once the state is initialised, and its logarithms and quotients are 450 of the 630 FP64 instructions
+// of a step's node (64 issue slots each).  512 x 400 with fields: 20 steps and their read-outs
+// 4.78 -> 1.50 ms; FP32 handles form their tables in less time than 144 B take.
+__global__ void __launch_bounds__(THREADS2) k_tables2(const float* __restrict__ u2, double* __restrict__ tab, size_t N) {
+  const size_t n = (size_t)blockIdx.x * THREADS2 + threadIdx.x;
+  if (n >= N) return;
+  Consts2<double> k;
+  node_tables2(k, (double)u2[n], (double)u2[N + n]);
+#pragma unroll
+  for (int i = 0; i < Q2; ++i) {
+    tab[(size_t)i * N + n] = k.E[i];
+    tab[(size_t)(Q2 + i) * N + n] = k.K3[i];
+    tab[(size_t)(2 * Q2 + i) * N + n] = k.L[i];
+    tab[(size_t)(3 * Q2 + i) * N + n] = k.M[i];
+  }
+}
+// Tables larger than this, or than the memory there is, are formed in every step instead.
+constexpr size_t TABLE_BYTES = 8ull << 30;
+
 int elementwise_blocks(size_t N) {
   return (int)std::min<size_t>((N + 255) / 256, 152 * 16);
 }
@@ -359,6 +393,7 @@ struct elbm2d_ctx {
   int cur = 0;
   void* T3 = nullptr;          // per-node T field (R), owned
   float* u2 = nullptr;         // per-node velocity [2][N], owned
+  double* tab = nullptr;       // its tables (FP64, k_tables2), owned, or null
   bool have_tensor = false, tensor_field = false;
   double D3[3] = {0, 0, 0};
   double u[2] = {0, 0};
@@ -456,7 +491,13 @@ cudaError_t launch_step2(elbm2d_ctx* h) {
   const int fb = h->params.fallback;
   auto kernel = pieces > 0 ? (vel == 2 ? k_step2<R, 2, true> : (vel == 1 ? k_step2<R, 1, true> : k_step2<R, 0, true>))
                            : (vel == 2 ? k_step2<R, 2, false> : (vel == 1 ? k_step2<R, 1, false> : k_step2<R, 0, false>));
-  return elbm::launch_next(kernel, grid, block, 0, h->stream, in, out, G, T3, h->u2, fb, h->d_counters, k);
+  const R* tab = nullptr;
+  if constexpr (std::is_same<R, double>::value) {
+    tab = h->tab;
+    if (vel == 2 && tab != nullptr) kernel = pieces > 0 ? k_step2<R, 3, true> : k_step2<R, 3, false>;
+  }
+  return elbm::launch_next(kernel, grid, block, 0, h->stream, in, out, G, T3, h->u2, tab, fb, h->d_counters,
+                           k);
 }
 
 elbm_status write_state(elbm2d_ctx* h, const void* in, elbm_dtype dt, int from_phi) {
@@ -573,6 +614,7 @@ void elbm2d_destroy(elbm2d_handle h) {
   cudaFree(h->pops[1]);
   cudaFree(h->T3);
   cudaFree(h->u2);
+  cudaFree(h->tab);
   cudaFree(h->d_counters);
   cudaFree(h->d_part);
   cudaFree(h->d_out4);
@@ -635,7 +677,9 @@ elbm_status elbm2d_set_velocity_uniform(elbm2d_handle h, const double u[2]) {
   if (h->u2) {
     CK2(cudaStreamSynchronize(h->stream), "sync");
     cudaFree(h->u2);
+    cudaFree(h->tab);
     h->u2 = nullptr;
+    h->tab = nullptr;
   }
   rebuild(h);
   return ELBM_OK;
@@ -654,11 +698,22 @@ elbm_status elbm2d_set_velocity_field(elbm2d_handle h, const float* u2) {
   CK2(cudaStreamSynchronize(h->stream), "sync");
   if (bad) {
     cudaFree(h->u2);
+    cudaFree(h->tab);
     h->u2 = nullptr;
+    h->tab = nullptr;
     return fail(h, ELBM_ERR_MACH, std::to_string(bad) + " nodes whose velocity gives a non-positive P_i(u)");
   }
   h->u[0] = h->u[1] = 0.0;
   rebuild(h);
+  const size_t bytes = 4 * Q2 * h->N * sizeof(double);
+  if (h->prec == 0 && h->tab == nullptr && bytes <= TABLE_BYTES && cudaMalloc((void**)&h->tab, bytes) != cudaSuccess) {
+    h->tab = nullptr;
+    cudaGetLastError();
+  }
+  if (h->tab != nullptr) {
+    k_tables2<<<(unsigned)((h->N + THREADS2 - 1) / THREADS2), THREADS2, 0, h->stream>>>(h->u2, h->tab, h->N);
+    CK2(cudaGetLastError(), "velocity tables");
+  }
   return ELBM_OK;
 }
 
