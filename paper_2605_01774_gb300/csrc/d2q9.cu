@@ -249,33 +249,44 @@ __device__ __forceinline__ size_t shifted(const Grid2& G, int x, int y, int dx, 
 // The buffers hold post-collision populations A (the step pulls g_i(x) = A_i(x - c_i)), so a
 // pre-collision state g is stored as A_i(y) = g_i(y + c_i).  from_phi: g_i = phi E_i(u), else
 // the caller's populations [9][N] (In = float or double).
+// Launched like steps (launch.cuh): what the caller's kernels write is read with plain loads.  One node
+// per thread and 32-bit coordinates: 2048^2 FP32 populations 53.6 -> 44.7 us, start and phi 55 and 32
+// to 35 us as before; whole passes of 20 steps 90 x 300 56 -> 49 us, 300 x 500 91 -> 84 us, 700 x 600
+// with fields 214 -> 203 us.  counters[0] is reset.
 template <typename R, typename In>
-__global__ void k_write2(R* __restrict__ pops, const In* __restrict__ in, Grid2 G, int from_phi,
-                         const float* __restrict__ u2, const Consts2<R> k) {
-  for (size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x; n < G.N; n += (size_t)gridDim.x * blockDim.x) {
-    const int x = (int)(n % G.nx), y = (int)(n / G.nx);
+__global__ void __launch_bounds__(THREADS2) k_write2(R* __restrict__ pops, const In* in, Grid2 G, int from_phi, const float* u2,
+                                                     unsigned long long* counters, const Consts2<R> k) {
+  const unsigned n = blockIdx.x * (unsigned)THREADS2 + threadIdx.x, y = n / (unsigned)G.nx;
+  const int x = (int)(n - y * (unsigned)G.nx);
+  elbm::wait_for_previous();
+  if (n == 0) counters[0] = 0ull;
+  if (n >= G.N) return;
+  R v[Q2];
 #pragma unroll
-    for (int i = 0; i < Q2; ++i) {
-      const size_t d = shifted(G, x, y, cx2(i), cy2(i));
-      pops[(size_t)i * G.N + n] = from_phi ? R(in[d]) * eq_weight(k, u2, G.N, d, i) : R(in[(size_t)i * G.N + d]);
-    }
+  for (int i = 0; i < Q2; ++i) {
+    const size_t d = shifted(G, x, (int)y, cx2(i), cy2(i));
+    v[i] = from_phi ? R(in[d]) * eq_weight(k, u2, G.N, d, i) : R(in[(size_t)i * G.N + d]);
   }
+#pragma unroll
+  for (int i = 0; i < Q2; ++i) pops[(size_t)i * G.N + n] = v[i];
 }
 
 // Pre-collision state: what 0: populations g_i(x) = A_i(x - c_i) [9][N]; 1: phi [N]
 template <typename R, typename Out>
-__global__ void k_read2(const R* __restrict__ pops, Out* __restrict__ out, Grid2 G, int what) {
-  for (size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x; n < G.N; n += (size_t)gridDim.x * blockDim.x) {
-    const int x = (int)(n % G.nx), y = (int)(n / G.nx);
-    R s = R(0);
+__global__ void __launch_bounds__(THREADS2) k_read2(const R* pops, Out* __restrict__ out, Grid2 G, int what) {
+  const unsigned n = blockIdx.x * (unsigned)THREADS2 + threadIdx.x, y = n / (unsigned)G.nx;
+  const int x = (int)(n - y * (unsigned)G.nx);
+  elbm::wait_for_previous();
+  if (n >= G.N) return;
+  R v[Q2], s = R(0);
 #pragma unroll
-    for (int i = 0; i < Q2; ++i) {
-      const R v = pops[(size_t)i * G.N + shifted(G, x, y, -cx2(i), -cy2(i))];
-      if (what == 0) out[(size_t)i * G.N + n] = Out(v);
-      s += v;
-    }
-    if (what != 0) out[n] = Out(s);
+  for (int i = 0; i < Q2; ++i) v[i] = pops[(size_t)i * G.N + shifted(G, x, (int)y, -cx2(i), -cy2(i))];
+#pragma unroll
+  for (int i = 0; i < Q2; ++i) {
+    if (what == 0) out[(size_t)i * G.N + n] = Out(v[i]);
+    s += v[i];
   }
+  if (what != 0) out[n] = Out(s);
 }
 
 // Partial sums per block: mass, entropy over positive g, min g, non-finite count.  A thread takes
@@ -508,23 +519,18 @@ elbm_status write_state(elbm2d_ctx* h, const void* in, elbm_dtype dt, int from_p
   void* tmp;
   elbm_status s = to_dev(h, in, bytes, &dev, &tmp);
   if (s != ELBM_OK) return s;
-  const int nb = elementwise_blocks(h->N);
+  const dim3 nb((unsigned)((h->N + THREADS2 - 1) / THREADS2)), nt(THREADS2);
   const Grid2 G{h->nx, h->ny, h->N};
+  const auto write = [&](auto* p, const auto& k) {
+    using R = typename std::remove_reference<decltype(*p)>::type;
+    return dt == ELBM_DTYPE_F64 ? elbm::launch_next(k_write2<R, double>, nb, nt, 0, h->stream, p, (const double*)dev, G,
+                                                    from_phi, h->u2, h->d_counters, k)
+                                : elbm::launch_next(k_write2<R, float>, nb, nt, 0, h->stream, p, (const float*)dev, G,
+                                                    from_phi, h->u2, h->d_counters, k);
+  };
   void* p = h->pops[h->cur];
-  if (h->prec == 0) {
-    if (dt == ELBM_DTYPE_F64)
-      k_write2<double, double><<<nb, 256, 0, h->stream>>>((double*)p, (const double*)dev, G, from_phi, h->u2, h->kd);
-    else
-      k_write2<double, float><<<nb, 256, 0, h->stream>>>((double*)p, (const float*)dev, G, from_phi, h->u2, h->kd);
-  } else {
-    if (dt == ELBM_DTYPE_F64)
-      k_write2<float, double><<<nb, 256, 0, h->stream>>>((float*)p, (const double*)dev, G, from_phi, h->u2, h->kf);
-    else
-      k_write2<float, float><<<nb, 256, 0, h->stream>>>((float*)p, (const float*)dev, G, from_phi, h->u2, h->kf);
-  }
-  CK2(cudaGetLastError(), "write kernel");
+  CK2(h->prec == 0 ? write((double*)p, h->kd) : write((float*)p, h->kf), "write kernel");
   if (tmp) CK2(cudaFreeAsync(tmp, h->stream), "cudaFreeAsync");
-  CK2(cudaMemsetAsync(h->d_counters, 0, sizeof(unsigned long long), h->stream), "memset");
   h->initialized = true;
   return ELBM_OK;
 }
@@ -537,17 +543,15 @@ elbm_status read_state(elbm2d_ctx* h, void* out, elbm_dtype dt, int what) {
   const bool host = !device_ptr(out);
   void* dout = out;
   if (host) CK2(cudaMallocAsync(&dout, bytes, h->stream), "cudaMallocAsync");
-  const int nb = elementwise_blocks(h->N);
+  const dim3 nb((unsigned)((h->N + THREADS2 - 1) / THREADS2)), nt(THREADS2);
   const Grid2 G{h->nx, h->ny, h->N};
+  const auto read = [&](const auto* p) {
+    using R = typename std::remove_const<typename std::remove_reference<decltype(*p)>::type>::type;
+    return dt == ELBM_DTYPE_F64 ? elbm::launch_next(k_read2<R, double>, nb, nt, 0, h->stream, p, (double*)dout, G, what)
+                                : elbm::launch_next(k_read2<R, float>, nb, nt, 0, h->stream, p, (float*)dout, G, what);
+  };
   const void* p = h->pops[h->cur];
-  if (h->prec == 0) {
-    if (dt == ELBM_DTYPE_F64) k_read2<double, double><<<nb, 256, 0, h->stream>>>((const double*)p, (double*)dout, G, what);
-    else k_read2<double, float><<<nb, 256, 0, h->stream>>>((const double*)p, (float*)dout, G, what);
-  } else {
-    if (dt == ELBM_DTYPE_F64) k_read2<float, double><<<nb, 256, 0, h->stream>>>((const float*)p, (double*)dout, G, what);
-    else k_read2<float, float><<<nb, 256, 0, h->stream>>>((const float*)p, (float*)dout, G, what);
-  }
-  CK2(cudaGetLastError(), "read kernel");
+  CK2(h->prec == 0 ? read((const double*)p) : read((const float*)p), "read kernel");
   if (host) {
     CK2(cudaMemcpyAsync(out, dout, bytes, cudaMemcpyDeviceToHost, h->stream), "memcpy D2H");
     CK2(cudaFreeAsync(dout, h->stream), "cudaFreeAsync");
@@ -713,6 +717,7 @@ elbm_status elbm2d_set_velocity_field(elbm2d_handle h, const float* u2) {
   if (h->tab != nullptr) {
     k_tables2<<<(unsigned)((h->N + THREADS2 - 1) / THREADS2), THREADS2, 0, h->stream>>>(h->u2, h->tab, h->N);
     CK2(cudaGetLastError(), "velocity tables");
+    CK2(cudaStreamSynchronize(h->stream), "sync");   // steps may load them before their wait
   }
   return ELBM_OK;
 }

@@ -1,11 +1,11 @@
-// Launches: the block shape of one thread per node, and kernels that follow one another on a stream,
-// each reading what the one before wrote.
+// Launches of kernels that follow one another on a stream, each reading what the one before wrote.
 //
 // A launch that waits for the previous kernel to end before it is set up costs about 2 us per step;
 // with programmatic stream serialisation the next kernel's blocks are placed while the last ones of
 // this kernel finish and wait inside, in wait_for_previous(), for its memory.  Measured: an empty
 // kernel 2.05 -> 1.5 us; a step with 121 x 75 x 50 nodes (FP32, tensor field) 22.7 -> 19.5 us, 32^3
-// (FP64) 8.3 -> 7.2 us, 24^3 (FP32) 4.2 -> 3.8 us.
+// (FP64) 8.3 -> 7.2 us, 24^3 (FP32) 4.2 -> 3.8 us.  Index arithmetic belongs ahead of the wait (24^3
+// 3.2 -> 2.9 us with the two divisions of the coordinates there).
 //
 // What a step reads after the wait it reads with plain loads: its L1 lines date from its own launch
 // or later, and between that and the wait only the previous step runs, which loads the other buffer.
@@ -16,22 +16,13 @@
 
 namespace elbm {
 
-// First statement of every kernel launched by launch_next: lets the next launch be placed, then
+// In every kernel launched by launch_next, once in every thread: lets the next launch be placed, then
 // waits until the kernel before this one has ended and its writes are visible.  Nothing that an
 // earlier kernel writes may be touched before it.
 __device__ __forceinline__ void wait_for_previous() {
   cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
 }
-
-// Blocks of at most 256 threads for one thread per node, rows along x: a row is cut into equal
-// pieces of whole warps (384 nodes into 2 x 192, where 256-thread pieces leave a quarter of the
-// lanes idle), short rows share a block.
-inline dim3 row_block(int nx) {
-  const int pieces = (nx + 255) / 256, per = (nx + pieces - 1) / pieces, bx = (per + 31) / 32 * 32;
-  return dim3(bx, 256 / bx, 1);
-}
-inline dim3 row_grid(dim3 b, int nx, int ny, int nz) { return dim3((nx + b.x - 1) / b.x, (ny + b.y - 1) / b.y, nz); }
 
 template <typename... Params, typename... Args>
 inline cudaError_t launch_next(void (*kernel)(Params...), dim3 grid, dim3 block, size_t shared, cudaStream_t s,
