@@ -158,12 +158,19 @@ __global__ void k_batch_write(const DomainInfo* dom, const int* tile_dom, const 
     const int rem = local - z * n * n;
     const int y = div_small(rem, n, d.inv_n);
     const int x = rem - y * n;
-    // equilibrium at u = 0 written so that the next pull sees g_i(x) = W_i phi0(x)
+    // equilibrium at u = 0 written so that the next pull sees g_i(x) = W_i phi0(x); neighbours by
+    // comparison (with three remainders by n for each of the 27 a start of the 512-box sweep took 3.69
+    // ms, now 3.44)
+    const int xs[3] = {x == 0 ? n - 1 : x - 1, x, x + 1 == n ? 0 : x + 1};
+    const int ys[3] = {(y == 0 ? n - 1 : y - 1) * n, y * n, (y + 1 == n ? 0 : y + 1) * n};
+    const int zs[3] = {(z == 0 ? n - 1 : z - 1) * n * n, z * n * n, (z + 1 == n ? 0 : z + 1) * n * n};
+    const float* const in = phi0 + d.off;
+    float* const out = buf + 27ll * d.off + local;
+    float p[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const int sx = (x + cx_of(i) + n) % n, sy = (y + cy_of(i) + n) % n, sz = (z + cz_of(i) + n) % n;
-      buf[27ll * d.off + (long long)i * N + local] = float(w_of(i)) * phi0[d.off + sx + n * (sy + n * sz)];
-    }
+    for (int i = 0; i < Q; ++i) p[i] = in[xs[cx_of(i) + 1] + ys[cy_of(i) + 1] + zs[cz_of(i) + 1]];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) out[(long long)i * N] = float(w_of(i)) * p[i];
   }
 }
 
