@@ -450,7 +450,7 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
                           mulq((int64_t)((uint64_t)az << sa), digits(Vz)) +
                           mulq((int64_t)((uint64_t)w << sa), digits(phi >> 3));
       int64_t kap;                                     // kappa 2^(sa - sh)
-      if (!half_quotient(num, den, 0x1p62f, kap)) return false;
+      if (!half_quotient(num, den, 0x1.fffep61f, kap)) return false;   // c below 2^63 - 2^43, sh >= 2
       c += sa == 0 ? kap : (kap + (1ll << (sa - 1))) >> sa;
     }
     const Q64 cq = digits(c);
@@ -502,7 +502,7 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
         }
       }
     }
-    if (mag >= 1u << 30) return false;
+    if (mag >= (1u << 30) - 1) return false;          // 2 d and its digits stay below 2^63
     if (second <= best * 1.0002f || nb < (1ll << 46)) {
 #pragma unroll 1
       for (int i = 0; i < Q; ++i) {
@@ -516,13 +516,16 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
         }
       }
     }
-    int64_t half = 0;                                 // alpha / 2, of 2 d
-    if (!half_quotient(nb, db, 0x1.1p63f, half)) return false;
+    // The blend starts at the nearer end, by the smaller one of alpha and 1 - alpha = -g*/d: half of
+    // that is at most 1/4, where alpha / 2 with alpha near 1 would reach the 2^63 that no int64_t holds.
+    const bool far = nb < db - nb;                    // alpha < 1/2: from g
+    int64_t half = 0;                                 // of 2 d
+    if (!half_quotient(far ? nb : db - nb, db, 0x1.1p62f, half)) return false;
     const Q64 aq = digits(half > 0 ? half : 0);
 #pragma unroll 1
     for (int i = 0; i < Q; ++i) {
-      const int64_t gi = keep.g(i);
-      keep.x(i) = gi - mulq(2 * (gi - keep.x(i)), aq);
+      const int64_t gi = keep.g(i), x = keep.x(i), m = mulq(2 * (gi - x), aq);
+      keep.x(i) = far ? gi - m : x + m;
     }
   }
 #pragma unroll 3
