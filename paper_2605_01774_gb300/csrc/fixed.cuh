@@ -88,6 +88,8 @@ inline FixConsts fix_consts(const Consts& k) {
   for (int q = 0; q < 6; ++q) f.quad[q] = q64_host(w0 * 4.5L * (ia[q] == ib[q] ? 1.0L : 2.0L) * u[ia[q]] * u[ib[q]]);
   for (int a = 0; a < 3; ++a) f.u[a] = q64_host(u[a]);
   const long double T[6] = {k.T.xx - 1.0L, k.T.xy, k.T.xz, k.T.yy - 1.0L, k.T.yz, k.T.zz - 1.0L};
+  for (int q = 0; q < 6; ++q) f.ok = f.ok && std::fabs((double)T[q]) < 1.5;   // not so where T is not finite
+  if (!f.ok) return f;
   for (int q = 0; q < 6; ++q) f.TmI[q] = q64_host(0.25L * T[q]);
   for (int i = 0; i < Q; ++i) {
     const long double s = 1.0L / (1 << (2 * nnz_of(i)));   // of 4^n dh_i
@@ -305,6 +307,16 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
   }
   const int etop = (int)(top >> 20);
   if (etop < 150 || etop > 1900) return false;       // also inf and NaN
+  if (Tn != nullptr) {
+    // T = 2I - S < 2, but rounds to 2 and a little above for D of 5e14 and more
+    uint32_t most = 0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const uint32_t h = (uint32_t)(bits_of(Tn[q]) >> 32) & 0x7fffffffu;
+      most = h > most ? h : most;
+    }
+    if (most >= 0x40000000u) return false;            // some |T| >= 2, or NaN
+  }
   const Q64 c49{1908874354, -954437177};             // 4/9
   int64_t phi, mx, my, mz;
   {

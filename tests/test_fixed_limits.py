@@ -1,5 +1,6 @@
 """The fixed-point FP64 collision (csrc/fixed.cuh, compiled for the host) where its numbers reach the
-ends of their range: at the onset of the positivity fallback."""
+ends of their range: at the onset of the positivity fallback, and at tensors that round to 2 and
+above."""
 import ctypes as C
 
 import numpy as np
@@ -66,3 +67,27 @@ def test_onset_of_the_fallback(lib, u):  # noqa: F811
         err = (np.abs(out.T - ref).max(0) / np.abs(pops).max(1)).astype(float)
         assert done.mean() > 0.98, beyond
         assert err[done].max() < 1e-13, beyond
+
+
+@pytest.mark.parametrize("u", [(0.0, 0.0, 0.0), (0.05, 0.03, 0.02)])
+def test_tensors_at_two(lib, u):  # noqa: F811
+    """T < 2 for every finite D, but T of D = 1e15 rounds to 2 and above: the node is left to FP64, as
+    are tensors that are not finite (uniform ones too); the largest T below 2 is taken, to 1e-13."""
+    u = np.array(u)
+    g = np.random.default_rng(11)
+    E = _equilibrium(u)
+    for bad in (2.0, np.nextafter(2.0, 3.0), -2.0, 4.0, 1e300, np.inf, np.nan):
+        T6 = _tensors(g, 12)
+        T6[np.arange(12), np.arange(12) // 2] = bad
+        pops = E * (1 + 5e-3 * g.standard_normal((12, 27)))
+        out, done, _ = _run(lib, pops, u, T6)
+        assert not done[1::2].any(), bad                 # odd nodes have tensors of their own
+        assert np.array_equal(out[1::2], pops[1::2])
+        assert np.isfinite(bad) or not done[::2].any()
+    T6 = _tensors(g, 6)
+    T6[np.arange(6), [0, 0, 3, 3, 5, 5]] = np.nextafter(2.0, 0.0)
+    pops = E * (1 + 5e-3 * g.standard_normal((6, 27)))
+    ref, _ = _collide(pops.T.astype(np.longdouble), u, _full(T6), THETA, 1)
+    out, done, _ = _run(lib, pops, u, T6)
+    assert done.all()
+    assert (np.abs(out.T - ref).max(0) / pops.max(1)).max() < 1e-13
