@@ -536,8 +536,10 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
     const Q64 aq = digits(half > 0 ? half : 0);
 #pragma unroll 1
     for (int i = 0; i < Q; ++i) {
-      const int64_t gi = keep.g(i), x = keep.x(i), m = mulq(2 * (gi - x), aq);
-      keep.x(i) = far ? gi - m : x + m;
+      const int64_t gi = keep.g(i), x = keep.x(i), m = mulq(2 * (gi - x), aq), b = far ? gi - m : x + m;
+      // the deciding population becomes 0, not a unit below: whole units of opposite sign meet and
+      // cancel where a plume's surroundings are empty, and 1/phi then overflows
+      keep.x(i) = gi >= 0 && b < 0 ? 0 : b;
     }
   }
 #pragma unroll 3

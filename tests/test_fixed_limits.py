@@ -1,6 +1,6 @@
 """The fixed-point FP64 collision (csrc/fixed.cuh, compiled for the host) where its numbers reach the
-ends of their range: at the onset of the positivity fallback, and at tensors that round to 2 and
-above."""
+ends of their range: at the onset of the positivity fallback, where it leaves a population at zero, and
+at tensors that round to 2 and above."""
 import ctypes as C
 
 import numpy as np
@@ -91,3 +91,15 @@ def test_tensors_at_two(lib, u):  # noqa: F811
     out, done, _ = _run(lib, pops, u, T6)
     assert done.all()
     assert (np.abs(out.T - ref).max(0) / pops.max(1)).max() < 1e-13
+
+
+@pytest.mark.parametrize("u", [(0.0, 0.0, 0.0), (0.05, 0.03, 0.02)])
+def test_fallback_leaves_nothing_negative(lib, u):  # noqa: F811
+    """Populations that are not negative stay so, exactly: the fallback's deciding one becomes 0."""
+    u = np.array(u)
+    g = np.random.default_rng(13)
+    n = 4000
+    pops, T6 = _equilibrium(u) * np.exp(1.0 * g.standard_normal((n, 27))), _tensors(g, n)
+    out, done, took = _run(lib, pops, u, T6)
+    assert (done & took).sum() > 200
+    assert out[done].min() >= 0.0
