@@ -229,9 +229,11 @@ k_adj_forward_fixed(const double* Gin, double* Gout, const double* __restrict__ 
     int x, y, z;
     coords(G, n, x, y, z);
     InShared<64> keep{kept + threadIdx.x};
-    if (!collide_fixed<1>(g, T, 0.0, false, true, c.fix, keep, took,
-                          [&](int i, double v) { Gout[i * G.N + nb(G, x, y, z, cx_of(i), cy_of(i), cz_of(i))] = v; }))
-      took = adj_node_f64(Gin, Gout, T6, G, n, c.pop);
+    const auto out = [&](int i, double v) { Gout[i * G.N + nb(G, x, y, z, cx_of(i), cy_of(i), cz_of(i))] = v; };
+    int etop;
+    const Fixed f = collide_fixed<1>(g, T, 0.0, false, true, c.fix, keep, took, etop, out);
+    if (f == Fixed::SMALL_ALPHA) blend_given(keep, etop, c.fix, out, [&](int i) { return Gin[i * G.N + n]; });
+    else if (f == Fixed::REFUSED) took = adj_node_f64(Gin, Gout, T6, G, n, c.pop);
   }
   const unsigned m = __ballot_sync(0xffffffffu, took);
   if (m && (threadIdx.x & 31) == 0) atomicAdd(fb, (unsigned long long)__popc(m));

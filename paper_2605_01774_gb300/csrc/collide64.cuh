@@ -17,7 +17,7 @@ struct StepConsts {};
 template <>
 struct StepConsts<FIXED> {
   FixConsts fix;
-  PopConsts<double> pop;   // for step_node_f64, which takes its address
+  PopConsts<double> pop;   // for step_node_f64 and pull_one, which take its address
 };
 
 template <int MODE, typename Launch>
@@ -47,26 +47,48 @@ __device__ __noinline__ bool step_node_f64(const Field<double>& in, const Grid& 
   return took;
 }
 
-// Collides g_i + r E_i (has_src false: r is 0), g the populations pulled into node n of the lattice G
+// Population i pulled into node n once more, with its source (src null: none); i not known at compile
+// time.
+static __device__ __noinline__ double pull_one(const Field<double>& in, const Grid& G, int n, int i, const float* src,
+                                               const PopConsts<double>& k) {
+  const int row = n / G.nx, x = n - row * G.nx, y = row % G.ny, z = row / G.ny;
+  const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+  double g;
+  if (G.dirichlet && ((cx == 1 && x == 0) || (cx == -1 && x == G.nx - 1))) {
+    g = 2.0 * w_of(i) * (x == 0 && cx == 1 ? k.phi_lo : k.phi_hi) - in.pops[(size_t)opp_of(i) * G.N + n];
+  } else {
+    const int sx = x < cx ? G.nx - 1 : (x - cx == G.nx ? 0 : x - cx);
+    const int sy = y < cy ? G.ny - 1 : (y - cy == G.ny ? 0 : y - cy);
+    const int sz = z < cz ? G.nz - 1 : (z - cz == G.nz ? 0 : z - cz);
+    g = in.pops[(size_t)i * G.N + (size_t)(sx + G.nx * (sy + G.ny * sz))];
+  }
+  return src != nullptr ? g + k.src_step * (double)src[n] * k.E[i] : g;
+}
+
+// Collides g_i + r E_i (src, the source field, null: r is 0), g the populations pulled into node n of the lattice G
 // from `in`, with the node's T where has_T, else the uniform one, and stores the result in `pout`,
 // `sout`.  Returns whether the positivity fallback was taken; proj as Storage::store returns it.
 // keep: where fixed point keeps the node's integers.
 template <typename R, int VEL, int MODE, typename Elem, typename Keep>
 __device__ __forceinline__ bool collide_and_store(R (&g)[Q], const Field<Elem>& in, Elem* __restrict__ pout,
                                                   float* __restrict__ sout, const Grid& G, int n, const Sym6<R>& T,
-                                                  bool has_T, R r, bool has_src, const PopConsts<R>& k,
+                                                  bool has_T, R r, const float* src, const PopConsts<R>& k,
                                                   const StepConsts<MODE>& c, bool fallback, Keep& keep, bool& proj,
                                                   const R* un = nullptr) {
   if constexpr (MODE == FIXED) {
     bool took;
+    int etop;
     const double t6[6] = {T.xx, T.xy, T.xz, T.yy, T.yz, T.zz};
     proj = false;
-    if (collide_fixed<VEL>(g, has_T ? t6 : nullptr, r, has_src, fallback, c.fix, keep, took,
-                           [&](int i, double v) { pout[(size_t)i * G.N + n] = v; }))
-      return took;
-    return step_node_f64<VEL>(in, G, n, T, r, has_src, c.pop, fallback, pout);
+    const auto out = [&](int i, double v) { pout[(size_t)i * G.N + n] = v; };
+    const Fixed f = collide_fixed<VEL>(g, has_T ? t6 : nullptr, r, src != nullptr, fallback, c.fix, keep, took, etop, out);
+    if (f == Fixed::SMALL_ALPHA)
+      blend_given(keep, etop, c.fix, out, [&](int i) { return pull_one(in, G, n, i, src, c.pop); });
+    else if (f == Fixed::REFUSED)
+      took = step_node_f64<VEL>(in, G, n, T, r, src != nullptr, c.pop, fallback, pout);
+    return took;
   } else {
-    if (has_src) {
+    if (src != nullptr) {
 #pragma unroll
       for (int i = 0; i < Q; ++i) g[i] += r * k.E[i];
     }

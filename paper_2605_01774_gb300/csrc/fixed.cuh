@@ -26,9 +26,9 @@
 // and the rest population takes what the rounding of the others leaves of phi, so that the
 // collision conserves the node's mass.
 //
-// collide_fixed returns false for a node that this cannot hold as well as FP64
-// does (non-finite or extreme values, phi small beside the largest 4^n_i g_i, a correction larger
-// than the node): the caller then pulls it again and runs the FP64 collision.
+// collide_fixed refuses a node that this cannot hold as well as FP64 does (non-finite or extreme
+// values, phi small beside the largest 4^n_i g_i, a correction larger than the node): the caller then
+// pulls it again and runs the FP64 collision.
 #pragma once
 #include <cmath>
 #include <cstdint>
@@ -38,8 +38,10 @@
 
 #ifdef __CUDACC__
 #define ELBM_HD __host__ __device__ __forceinline__
+#define ELBM_COLD __host__ __device__ __noinline__
 #else
 #define ELBM_HD inline
+#define ELBM_COLD inline
 #endif
 
 namespace elbm {
@@ -67,6 +69,7 @@ struct FixConsts {
   Q64 TmI[6];      // (T - I) / 4 of the uniform T = 2I - S
   Q64 K3[Q], L[Q], M[Q];   // 4^-n K3 / 8, 4^-n L, 16^-n M / 16
   uint32_t exponent[Q];    // (5 - 2 n) << 20 (from_fixed)
+  double E[Q];
   double theta2;
   bool ok;                 // the tables fit, and the positivity threshold is 0
 };
@@ -99,6 +102,7 @@ inline FixConsts fix_consts(const Consts& k) {
     f.L[i] = q64_host(s * k.L[i]);
     f.M[i] = q64_host(0.0625L * s * s * k.M[i]);
     f.exponent[i] = (uint32_t)(5 - 2 * nnz_of(i)) << 20;
+    f.E[i] = k.E[i];
   }
   f.theta2 = k.theta2;
   return f;
@@ -280,17 +284,70 @@ struct InShared {
   ELBM_HD int64_t& pair(int i) { return p[(2 * Q + i) * STRIDE]; }
 };
 
+// What collide_fixed did with a node: left it to FP64, collided it, or came to a fallback whose alpha
+// takes more bits than it kept (blend_given ends such a node).
+enum class Fixed { REFUSED, DONE, SMALL_ALPHA };
+
+// keep.x(i) from keep.g(i) towards keep.x(i) by alpha = 2^-63 half (far), or from keep.x(i) towards
+// keep.g(i) by 1 - alpha = 2^-63 half.
+template <typename Keep>
+ELBM_HD void blend(Keep& keep, int64_t half, bool far) {
+  const Q64 aq = digits(half > 0 ? half : 0);
+#pragma unroll 1
+  for (int i = 0; i < Q; ++i) {
+    const int64_t gi = keep.g(i), x = keep.x(i), m = mulq(2 * (gi - x), aq), b = far ? gi - m : x + m;
+    // the deciding population becomes 0, not a unit below: whole units of opposite sign meet and
+    // cancel where a plume's surroundings are empty, and 1/phi then overflows
+    keep.x(i) = gi >= 0 && b < 0 ? 0 : b;
+  }
+}
+
+// The results keep.x to out(i, value).
+template <typename Keep, typename Out>
+ELBM_HD void put(Keep& keep, int etop, const FixConsts& k, Out& out) {
+#pragma unroll 3
+  for (int i = 0; i < Q; ++i) {
+    const int64_t x = keep.x(i);
+    out(i, from_fixed((uint64_t)(x < 0 ? -x : x), (uint32_t)(x >> 32) & 0x80000000u, k.exponent[i] + ((uint32_t)etop << 20)));
+  }
+}
+
+// The fallback of a node whose deciding d is less than 1/16 of the largest: a unit of its g moves the
+// other populations by more than 16 units, where FP64 arithmetic knows a g that is small beside the
+// others to its last bit.  So alpha is formed in FP64 from given(i), population i as collide_fixed got
+// it, with its source.  Out of line and ended here: with its loop in collide_fixed the step of the
+// driven 128^3 box, which never comes here, took 12.5 instead of 7.7 ms (12 steps and read-outs).
+template <typename Keep, typename Out, typename Given>
+ELBM_COLD void blend_given(Keep& keep, int etop, const FixConsts& k, Out out, Given given) {
+  const double unit = value_of((uint64_t)(2103 - etop) << 52);
+  double num = 1.0, den = 1.0;                        // alpha
+#pragma unroll 1
+  for (int i = 0; i < Q; ++i) {
+    const int64_t gi = keep.g(i), x = keep.x(i);
+    if (x < 0 && gi > x) {
+      const double g = given(i), n = g > 0.0 ? g * (double)(1 << (2 * nnz_of(i))) * unit : 0.0, d = n - (double)x;
+      if (n * den < num * d) {
+        num = n;
+        den = d;
+      }
+    }
+  }
+  const bool far = num < 0.5 * den;
+  blend(keep, (int64_t)((far ? num : den - num) / den * 0x1p63), far);
+  put(keep, etop, k, out);
+}
+
 // One node.  v: the 27 pre-collision populations.  Tn: the node's T, or null for the uniform one.
 // src: source term r, g_i + r E_i is collided (0: none).  keep: storage for the node's integers.
-// out(i, value): receives the post-collision populations (only where it returns true).
-// took: the positivity fallback (threshold 0) was taken.
+// out(i, value): receives the post-collision populations (only of a node that is DONE).
+// took: the positivity fallback (threshold 0) was taken.  etop: what blend_given needs besides keep.
 //
 // The loops with products and conversions are not unrolled: unrolled, the collision is about 90 KB
 // of instructions that every warp runs through once, and fetching them, not executing them, sets
 // the pace (ncu: 2.6 to 4.6 warps per issue stalled for want of instructions).
 template <int VEL, typename Keep, typename Out>
-ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, bool has_src, bool fallback,
-                           const FixConsts& k, Keep& keep, bool& took, Out out) {
+ELBM_HD Fixed collide_fixed(const double (&v)[Q], const double* Tn, double src, bool has_src, bool fallback,
+                            const FixConsts& k, Keep& keep, bool& took, int& etop, Out out) {
   took = false;
   uint32_t top = 0, sign = 0;
 #pragma unroll
@@ -305,8 +362,8 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
     top = a > top ? a : top;
     sign |= h;
   }
-  const int etop = (int)(top >> 20);
-  if (etop < 150 || etop > 1900) return false;       // also inf and NaN
+  etop = (int)(top >> 20);
+  if (etop < 150 || etop > 1900) return Fixed::REFUSED;       // also inf and NaN
   if (Tn != nullptr) {
     // T = 2I - S < 2, but rounds to 2 and a little above for D of 5e14 and more
     uint32_t most = 0;
@@ -315,7 +372,7 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
       const uint32_t h = (uint32_t)(bits_of(Tn[q]) >> 32) & 0x7fffffffu;
       most = h > most ? h : most;
     }
-    if (most >= 0x40000000u) return false;            // some |T| >= 2, or NaN
+    if (most >= 0x40000000u) return Fixed::REFUSED;            // some |T| >= 2, or NaN
   }
   const Q64 c49{1908874354, -954437177};             // 4/9
   int64_t phi, mx, my, mz;
@@ -361,13 +418,13 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
     my = weigh(0, d[2], (d[1] + d[3]) + (d[11] - d[5]), (d[10] - d[4]) + (d[12] - d[6]));
     mz = weigh(0, d[0], (d[3] - d[1]) + (d[9] - d[7]), (d[6] - d[4]) + (d[12] - d[10]));
     // phi below t/8 to t/4: the units would be coarse beside it
-    if (phi < (1ll << 55)) return false;
+    if (phi < (1ll << 55)) return Fixed::REFUSED;
     if (VEL != 0) {
       if ((int32_t)sign < 0) {
         int64_t c[4] = {0, 0, 0, 0};
 #pragma unroll
         for (int i = 0; i < Q; ++i) c[nnz_of(i)] -= G[i] < 0 ? G[i] : 0;
-        if (phi < (weigh(c[0], c[1], c[2], c[3]) >> 3)) return false;
+        if (phi < (weigh(c[0], c[1], c[2], c[3]) >> 3)) return Fixed::REFUSED;
       }
       // X: 4^n dh
       const Q64 f = digits(phi);
@@ -427,7 +484,7 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
       const int64_t x = keep.x(i);
       mag |= (uint32_t)((int32_t)(x >> 32) ^ (int32_t)(x >> 63));
     }
-    if (mag >= 1u << 28) return false;
+    if (mag >= 1u << 28) return Fixed::REFUSED;
     const int sh = mag == 0 ? 30 : clz32(mag) - 2;
     // kappa 2^-sh = num / (2 den), num = sum dh (K3 c.a + L phi) / 8, den = sum dh^2 M / 16
     int64_t Vx = 0, Vy = 0, Vz = 0, w, den;
@@ -462,7 +519,7 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
                           mulq((int64_t)((uint64_t)az << sa), digits(Vz)) +
                           mulq((int64_t)((uint64_t)w << sa), digits(phi >> 3));
       int64_t kap;                                     // kappa 2^(sa - sh)
-      if (!half_quotient(num, den, 0x1.fffep61f, kap)) return false;   // c below 2^63 - 2^43, sh >= 2
+      if (!half_quotient(num, den, 0x1.fffep61f, kap)) return Fixed::REFUSED;   // c below 2^63 - 2^43, sh >= 2
       c += sa == 0 ? kap : (kap + (1ll << (sa - 1))) >> sa;
     }
     const Q64 cq = digits(c);
@@ -502,7 +559,8 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
 #pragma unroll 1
     for (int i = 0; i < Q; ++i) {
       const int64_t gi = keep.g(i), x = keep.x(i), dd = gi - x;
-      mag |= (uint32_t)((int32_t)(dd >> 32) ^ (int32_t)(dd >> 63));
+      const uint32_t size = (uint32_t)((int32_t)(dd >> 32) ^ (int32_t)(dd >> 63));
+      mag = size > mag ? size : mag;
       if (x < 0 && dd > 0) {
         const int64_t n = gi > 0 ? gi : 0;
         const float q = quotient((float)(int32_t)(n >> 32), (float)(int32_t)(dd >> 32) + 1.0f);
@@ -514,7 +572,7 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
         }
       }
     }
-    if (mag >= (1u << 30) - 1) return false;          // 2 d and its digits stay below 2^63
+    if (mag >= (1u << 30) - 1) return Fixed::REFUSED;          // 2 d and its digits stay below 2^63
     if (second <= best * 1.0002f || nb < (1ll << 46)) {
 #pragma unroll 1
       for (int i = 0; i < Q; ++i) {
@@ -528,26 +586,27 @@ ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, b
         }
       }
     }
+    if ((uint32_t)(db >> 28) < mag) return Fixed::SMALL_ALPHA;
     // The blend starts at the nearer end, by the smaller one of alpha and 1 - alpha = -g*/d: half of
     // that is at most 1/4, where alpha / 2 with alpha near 1 would reach the 2^63 that no int64_t holds.
     const bool far = nb < db - nb;                    // alpha < 1/2: from g
-    int64_t half = 0;                                 // of 2 d
-    if (!half_quotient(far ? nb : db - nb, db, 0x1.1p62f, half)) return false;
-    const Q64 aq = digits(half > 0 ? half : 0);
-#pragma unroll 1
-    for (int i = 0; i < Q; ++i) {
-      const int64_t gi = keep.g(i), x = keep.x(i), m = mulq(2 * (gi - x), aq), b = far ? gi - m : x + m;
-      // the deciding population becomes 0, not a unit below: whole units of opposite sign meet and
-      // cancel where a plume's surroundings are empty, and 1/phi then overflows
-      keep.x(i) = gi >= 0 && b < 0 ? 0 : b;
-    }
+    int64_t half = 0;
+    if (!half_quotient(far ? nb : db - nb, db, 0x1.1p62f, half)) return Fixed::REFUSED;
+    blend(keep, half, far);
   }
-#pragma unroll 3
-  for (int i = 0; i < Q; ++i) {
-    const int64_t x = keep.x(i);
-    out(i, from_fixed((uint64_t)(x < 0 ? -x : x), (uint32_t)(x >> 32) & 0x80000000u, k.exponent[i] + ((uint32_t)etop << 20)));
-  }
-  return true;
+  put(keep, etop, k, out);
+  return Fixed::DONE;
+}
+
+// The whole collision where v still holds the populations as given; false for a node left to FP64.
+template <int VEL, typename Keep, typename Out>
+ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, bool has_src, bool fallback,
+                           const FixConsts& k, Keep& keep, bool& took, Out out) {
+  int etop;
+  const Fixed f = collide_fixed<VEL>(v, Tn, src, has_src, fallback, k, keep, took, etop, out);
+  if (f == Fixed::SMALL_ALPHA)
+    blend_given(keep, etop, k, out, [&](int i) { return v[i] + (has_src ? src * k.E[i] : 0.0); });
+  return f != Fixed::REFUSED;
 }
 
 }  // namespace elbm

@@ -60,10 +60,10 @@ k_step(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G
     if constexpr (MODE == FIXED) keep = Kept<MODE>{kept + threadIdx.x};
     if constexpr (VEL == 2) {
       const R un[3] = {R(__ldg(u3 + n)), R(__ldg(u3 + G.N + n)), R(__ldg(u3 + 2 * G.N + n))};
-      took = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, c,
+      took = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, c,
                                              fallback != 0, keep, proj, un);
     } else {
-      took = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, c,
+      took = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, c,
                                              fallback != 0, keep, proj);
     }
   }

@@ -383,10 +383,10 @@ k_step_rows(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
       bool t, pr;
       if constexpr (VEL == 2) {
         const R un[3] = {R(__ldg(u3 + n)), R(__ldg(u3 + G.N + n)), R(__ldg(u3 + 2 * G.N + n))};
-        t = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, kc,
+        t = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, kc,
                                             fallback != 0, keep, pr, un);
       } else {
-        t = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, kc,
+        t = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, kc,
                                             fallback != 0, keep, pr);
       }
       took += t ? 1u : 0u;
@@ -609,10 +609,10 @@ k_step_pipe(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
       bool tk, pr;
       if constexpr (VEL == 2) {
         const R un[3] = {R(__ldg(u3 + n)), R(__ldg(u3 + G.N + n)), R(__ldg(u3 + 2 * G.N + n))};
-        tk = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, kc,
+        tk = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, kc,
                                              fallback != 0, keep, pr, un);
       } else {
-        tk = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src != nullptr, k, kc,
+        tk = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, kc,
                                              fallback != 0, keep, pr);
       }
       took += tk ? 1u : 0u;

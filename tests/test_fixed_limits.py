@@ -1,6 +1,6 @@
 """The fixed-point FP64 collision (csrc/fixed.cuh, compiled for the host) where its numbers reach the
-ends of their range: at the onset of the positivity fallback, where it leaves a population at zero, and
-at tensors that round to 2 and above."""
+ends of their range: at the onset of the positivity fallback, where it leaves a population at zero, where a
+small population decides it, and at tensors that round to 2 and above."""
 import ctypes as C
 
 import numpy as np
@@ -103,3 +103,23 @@ def test_fallback_leaves_nothing_negative(lib, u):  # noqa: F811
     out, done, took = _run(lib, pops, u, T6)
     assert (done & took).sum() > 200
     assert out[done].min() >= 0.0
+
+
+@pytest.mark.parametrize("u", [(0.0, 0.0, 0.0), (0.05, 0.03, 0.02)])
+@pytest.mark.parametrize("spread", [2.0, 4.0, 8.0])
+def test_small_deciding_populations(lib, spread, u):  # noqa: F811
+    """Populations that differ by decades, of which a small one often decides the fallback: no further
+    from the exact collision than FP64 arithmetic is (root mean square over the nodes, relative to the
+    largest population)."""
+    u = np.array(u)
+    g = np.random.default_rng(17)
+    n = 40000
+    pops, T6 = _equilibrium(u) * np.exp(spread * g.standard_normal((n, 27))), _tensors(g, n)
+    out, done, took = _run(lib, pops, u, T6)
+    assert (done & took).sum() > 1000
+    pops, T6, out = pops[done], T6[done], out[done]
+    ref, fb = _collide(pops.T.astype(np.longdouble), u, _full(T6), THETA, 1)
+    assert np.array_equal(fb, took[done])
+    f64 = _collide(pops.T, u, _full(T6), THETA, 1)[0]
+    rms = lambda x: float(np.sqrt(((np.abs(x - ref).max(0) / pops.max(1)) ** 2).mean()))  # noqa: E731
+    assert rms(out.T) <= rms(f64), (rms(out.T), rms(f64))
