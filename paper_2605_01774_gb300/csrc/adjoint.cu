@@ -192,7 +192,7 @@ k_adj_forward(const R* Gin, R* Gout, const R* __restrict__ T6, AGrid G, const Po
   if (m && (threadIdx.x & 31) == 0) atomicAdd(fb, (unsigned long long)__popc(m));
 }
 
-// One of the few nodes that fixed point cannot hold, out of line.
+// A node left to FP64 (collide64.cuh), out of line.
 __device__ __noinline__ bool adj_node_f64(const double* Gin, double* Gout, const double* T6, const AGrid& G, int n,
                                           const PopConsts<double>& k) {
   double g[Q], phi;
@@ -219,6 +219,7 @@ k_adj_forward_fixed(const double* Gin, double* Gout, const double* __restrict__ 
   __shared__ int64_t kept[KEPT * 64];
   wait_for_previous();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  const Lanes lanes{__ballot_sync(0xffffffffu, n < G.N), G.nx};
   bool took = false;
   if (n < G.N) {
     double g[Q], T[6];
@@ -231,7 +232,9 @@ k_adj_forward_fixed(const double* Gin, double* Gout, const double* __restrict__ 
     InShared<64> keep{kept + threadIdx.x};
     const auto out = [&](int i, double v) { Gout[i * G.N + nb(G, x, y, z, cx_of(i), cy_of(i), cz_of(i))] = v; };
     int etop;
-    const Fixed f = collide_fixed<1>(g, T, 0.0, false, true, c.fix, keep, took, etop, out);
+    const Fixed f = collide_fixed<1>(g, T, 0.0, false, true, c.fix, keep, took, etop, out,
+                                     [&](bool refuse) { return lanes.any(refuse); });
+    __syncwarp(lanes.all);
     if (f == Fixed::SMALL_ALPHA) blend_given(keep, etop, c.fix, out, [&](int i) { return Gin[i * G.N + n]; });
     else if (f == Fixed::REFUSED) took = adj_node_f64(Gin, Gout, T6, G, n, c.pop);
   }

@@ -319,12 +319,20 @@ ELBM_HD void put(Keep& keep, int etop, const FixConsts& k, Out& out) {
 // driven 128^3 box, which never comes here, took 12.5 instead of 7.7 ms (12 steps and read-outs).
 template <typename Keep, typename Out, typename Given>
 ELBM_COLD void blend_given(Keep& keep, int etop, const FixConsts& k, Out out, Given given) {
+  // Only populations whose kept digits leave it open decide; the others need not be fetched again.
+  float most = 1.0f;
+#pragma unroll 1
+  for (int i = 0; i < Q; ++i) {
+    const int64_t gi = keep.g(i), x = keep.x(i);
+    if (x < 0 && gi > x) most = fminf(most, quotient((float)(gi > 0 ? gi : 0) + 2.0f, (float)(gi - x)));
+  }
+  most *= 1.001f;
   const double unit = value_of((uint64_t)(2103 - etop) << 52);
   double num = 1.0, den = 1.0;                        // alpha
 #pragma unroll 1
   for (int i = 0; i < Q; ++i) {
     const int64_t gi = keep.g(i), x = keep.x(i);
-    if (x < 0 && gi > x) {
+    if (x < 0 && gi > x && (float)gi - 2.0f <= most * ((float)(gi - x) + 2.0f)) {
       const double g = given(i), n = g > 0.0 ? g * (double)(1 << (2 * nnz_of(i))) * unit : 0.0, d = n - (double)x;
       if (n * den < num * d) {
         num = n;
@@ -341,13 +349,14 @@ ELBM_COLD void blend_given(Keep& keep, int etop, const FixConsts& k, Out out, Gi
 // src: source term r, g_i + r E_i is collided (0: none).  keep: storage for the node's integers.
 // out(i, value): receives the post-collision populations (only of a node that is DONE).
 // took: the positivity fallback (threshold 0) was taken.  etop: what blend_given needs besides keep.
+// vote(refuse): whether the node is refused, where it would be by itself or not.
 //
 // The loops with products and conversions are not unrolled: unrolled, the collision is about 90 KB
 // of instructions that every warp runs through once, and fetching them, not executing them, sets
 // the pace (ncu: 2.6 to 4.6 warps per issue stalled for want of instructions).
-template <int VEL, typename Keep, typename Out>
+template <int VEL, typename Keep, typename Out, typename Vote>
 ELBM_HD Fixed collide_fixed(const double (&v)[Q], const double* Tn, double src, bool has_src, bool fallback,
-                            const FixConsts& k, Keep& keep, bool& took, int& etop, Out out) {
+                            const FixConsts& k, Keep& keep, bool& took, int& etop, Out out, Vote vote) {
   took = false;
   uint32_t top = 0, sign = 0;
 #pragma unroll
@@ -363,17 +372,7 @@ ELBM_HD Fixed collide_fixed(const double (&v)[Q], const double* Tn, double src, 
     sign |= h;
   }
   etop = (int)(top >> 20);
-  if (etop < 150 || etop > 1900) return Fixed::REFUSED;       // also inf and NaN
-  if (Tn != nullptr) {
-    // T = 2I - S < 2, but rounds to 2 and a little above for D of 5e14 and more
-    uint32_t most = 0;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const uint32_t h = (uint32_t)(bits_of(Tn[q]) >> 32) & 0x7fffffffu;
-      most = h > most ? h : most;
-    }
-    if (most >= 0x40000000u) return Fixed::REFUSED;            // some |T| >= 2, or NaN
-  }
+  bool refuse = etop < 150 || etop > 1900;           // also inf and NaN
   const Q64 c49{1908874354, -954437177};             // 4/9
   int64_t phi, mx, my, mz;
   {
@@ -406,10 +405,6 @@ ELBM_HD Fixed collide_fixed(const double (&v)[Q], const double* Tn, double src, 
         }
       }
     }
-    if (VEL != 0 || fallback) {
-#pragma unroll
-      for (int i = 0; i < Q; ++i) keep.g(i) = G[i];
-    }
     // moments, by classes of 1, 2 and 3 nonzero components (d: the odd part of each pair)
 #pragma unroll
     for (int i = 14; i < Q; ++i) d[i - 14] = G[i] - G[26 - i];
@@ -418,14 +413,20 @@ ELBM_HD Fixed collide_fixed(const double (&v)[Q], const double* Tn, double src, 
     my = weigh(0, d[2], (d[1] + d[3]) + (d[11] - d[5]), (d[10] - d[4]) + (d[12] - d[6]));
     mz = weigh(0, d[0], (d[3] - d[1]) + (d[9] - d[7]), (d[6] - d[4]) + (d[12] - d[10]));
     // phi below t/8 to t/4: the units would be coarse beside it
-    if (phi < (1ll << 55)) return Fixed::REFUSED;
-    if (VEL != 0) {
-      if ((int32_t)sign < 0) {
-        int64_t c[4] = {0, 0, 0, 0};
+    refuse |= phi < (1ll << 55);
+    if (VEL != 0 && (int32_t)sign < 0) {
+      int64_t c[4] = {0, 0, 0, 0};
 #pragma unroll
-        for (int i = 0; i < Q; ++i) c[nnz_of(i)] -= G[i] < 0 ? G[i] : 0;
-        if (phi < (weigh(c[0], c[1], c[2], c[3]) >> 3)) return Fixed::REFUSED;
-      }
+      for (int i = 0; i < Q; ++i) c[nnz_of(i)] -= G[i] < 0 ? G[i] : 0;
+      refuse |= phi < (weigh(c[0], c[1], c[2], c[3]) >> 3);
+    }
+    // nearly all refusals are known here, at a tenth of the collision's instructions
+    if (vote(refuse)) return Fixed::REFUSED;
+    if (VEL != 0 || fallback) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) keep.g(i) = G[i];
+    }
+    if (VEL != 0) {
       // X: 4^n dh
       const Q64 f = digits(phi);
       int64_t B[6], e[13];
@@ -452,6 +453,16 @@ ELBM_HD Fixed collide_fixed(const double (&v)[Q], const double* Tn, double src, 
   // a = (T - I) j
   int64_t ax, ay, az;
   {
+    if (Tn != nullptr) {
+      // T = 2I - S < 2, but rounds to 2 and a little above for D of 5e14 and more
+      uint32_t most = 0;
+#pragma unroll
+      for (int q = 0; q < 6; ++q) {
+        const uint32_t h = (uint32_t)(bits_of(Tn[q]) >> 32) & 0x7fffffffu;
+        most = h > most ? h : most;
+      }
+      if (most >= 0x40000000u) return Fixed::REFUSED;   // some |T| >= 2, or NaN
+    }
     Q64 T[6];
 #pragma unroll
     for (int q = 0; q < 6; ++q)
@@ -572,7 +583,7 @@ ELBM_HD Fixed collide_fixed(const double (&v)[Q], const double* Tn, double src, 
         }
       }
     }
-    if (mag >= (1u << 30) - 1) return Fixed::REFUSED;          // 2 d and its digits stay below 2^63
+    if (mag >= (1u << 30) - 1) return Fixed::REFUSED;   // 2 d and its digits stay below 2^63
     if (second <= best * 1.0002f || nb < (1ll << 46)) {
 #pragma unroll 1
       for (int i = 0; i < Q; ++i) {
@@ -603,7 +614,8 @@ template <int VEL, typename Keep, typename Out>
 ELBM_HD bool collide_fixed(const double (&v)[Q], const double* Tn, double src, bool has_src, bool fallback,
                            const FixConsts& k, Keep& keep, bool& took, Out out) {
   int etop;
-  const Fixed f = collide_fixed<VEL>(v, Tn, src, has_src, fallback, k, keep, took, etop, out);
+  const Fixed f = collide_fixed<VEL>(v, Tn, src, has_src, fallback, k, keep, took, etop, out,
+                                     [](bool refuse) { return refuse; });
   if (f == Fixed::SMALL_ALPHA)
     blend_given(keep, etop, k, out, [&](int i) { return v[i] + (has_src ? src * k.E[i] : 0.0); });
   return f != Fixed::REFUSED;

@@ -22,22 +22,28 @@ constexpr int THREADS = 64;
 #define ELBM_STEP_MINB 3
 #endif
 // FP64 in fixed point: 34 KB of shared memory per 64 nodes (fixed.cuh) lets 6 blocks stand on an SM
-// at 168 registers.  Measured on the 96 x 80 x 72 plume, 20 steps and their read-outs: 4 blocks 4.09,
-// 6 blocks 3.69 ms; all loops unrolled, no shared memory, 2 to 4 blocks of 128 3.97 to 4.24 ms
+// at 168 registers.  Measured on the 96 x 80 x 72 plume, 20 steps and their read-outs: 4 blocks 4.02,
+// 6 blocks 3.54 ms; all loops unrolled, no shared memory, 2 to 4 blocks of 128 3.97 to 4.24 ms
 // (waiting for instructions); FP64 arithmetic 10.7 ms.
+// FEW: lattices whose blocks stand on the chip 4 to an SM take the registers that 6 would not leave
+// them; their time is a node's chain, not throughput.  A step of 32^3 nodes with a plume two nodes
+// wide (mostly left to FP64) 77 -> 53 us (FP64 arithmetic alone 54), 5.3 wide 18.5 -> 15 us; 40^3, 6.6
+// blocks to an SM, takes 127 us (4 blocks) and 129 us, later 122 and 102 us.
 #ifndef ELBM_FIXED_MINB
 #define ELBM_FIXED_MINB 6
 #endif
-template <typename Elem, int MODE>
+constexpr int FEW_PER_SM = 4;
+constexpr size_t FEW_NODES = 152ull * FEW_PER_SM * THREADS;
+template <typename Elem, int MODE, bool FEW>
 __host__ __device__ constexpr int step_blocks() {
-  return MODE == FIXED ? ELBM_FIXED_MINB : (std::is_same<Elem, double>::value ? 1 : ELBM_STEP_MINB) * (256 / THREADS);
+  return MODE == FIXED ? (FEW ? FEW_PER_SM : ELBM_FIXED_MINB) : (std::is_same<Elem, double>::value ? 1 : ELBM_STEP_MINB) * (256 / THREADS);
 }
 
 template <int MODE>
 using Kept = typename std::conditional<MODE == FIXED, InShared<THREADS>, KeepNone>::type;
 
-template <typename Elem, int VEL, int MODE>
-__global__ void __launch_bounds__(THREADS, step_blocks<Elem, MODE>())
+template <typename Elem, int VEL, int MODE, bool FEW>
+__global__ void __launch_bounds__(THREADS, step_blocks<Elem, MODE, FEW>())
 k_step(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G,
        const typename Storage<Elem>::real* __restrict__ T6,
        const float* __restrict__ src, const float* __restrict__ u3, int fallback,
@@ -49,6 +55,8 @@ k_step(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G
   __shared__ int64_t kept[MODE == FIXED ? KEPT * THREADS : 1];
   wait_for_previous();
   bool took = false, proj = false;
+  Lanes lanes{};
+  if constexpr (MODE == FIXED) lanes = Lanes{__ballot_sync(0xffffffffu, z < G.nz), G.nx};
   if (z < G.nz) {
     const int n = (int)m;
     R g[Q];
@@ -61,10 +69,10 @@ k_step(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, Grid G
     if constexpr (VEL == 2) {
       const R un[3] = {R(__ldg(u3 + n)), R(__ldg(u3 + G.N + n)), R(__ldg(u3 + 2 * G.N + n))};
       took = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, c,
-                                             fallback != 0, keep, proj, un);
+                                             fallback != 0, lanes, keep, proj, un);
     } else {
       took = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, c,
-                                             fallback != 0, keep, proj);
+                                             fallback != 0, lanes, keep, proj);
     }
   }
   // one counter update per block
@@ -84,7 +92,11 @@ static cudaError_t launch_t(const StepLaunch& L, cudaStream_t s) {
   const PopConsts<R>& k = *reinterpret_cast<const PopConsts<R>*>(std::is_same<R, double>::value ? (const void*)L.kd
                                                                                                : (const void*)L.kf);
   const dim3 blocks((unsigned)((L.N + THREADS - 1) / THREADS));
-  return launch_next(k_step<Elem, VEL, MODE>, blocks, dim3(THREADS), 0, s, in, static_cast<Elem*>(L.pout), L.sout, G,
+  auto kernel = k_step<Elem, VEL, MODE, false>;
+  if constexpr (MODE == FIXED) {
+    if (L.N <= FEW_NODES) kernel = k_step<Elem, VEL, MODE, true>;
+  }
+  return launch_next(kernel, blocks, dim3(THREADS), 0, s, in, static_cast<Elem*>(L.pout), L.sout, G,
                      static_cast<const R*>(L.T6), L.src, L.u3, L.fallback, L.counters, k, step_consts<MODE>(L));
 }
 

@@ -375,6 +375,8 @@ k_step_rows(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
           issue_desc(s_desc[cfirst], yz.x, yz.y, G, smem + s * SB, &full[s]);
         }
       }
+      Lanes lanes{};
+      if constexpr (MODE == FIXED) lanes = Lanes{__ballot_sync(0xffffffffu, valid), G.nx};
       if (!valid) continue;
       if (G.dirichlet) abb_faces<Elem, R>(g, in, G, x, n, k);
       // merged Strang half-steps of consecutive steps (Section 3.3)
@@ -384,10 +386,10 @@ k_step_rows(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
       if constexpr (VEL == 2) {
         const R un[3] = {R(__ldg(u3 + n)), R(__ldg(u3 + G.N + n)), R(__ldg(u3 + 2 * G.N + n))};
         t = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, kc,
-                                            fallback != 0, keep, pr, un);
+                                            fallback != 0, lanes, keep, pr, un);
       } else {
         t = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, kc,
-                                            fallback != 0, keep, pr);
+                                            fallback != 0, lanes, keep, pr);
       }
       took += t ? 1u : 0u;
       proj += pr ? 1u : 0u;
@@ -586,7 +588,7 @@ k_step_pipe(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
     if (lane == 0) it = atomicAdd(&s_item, 1);
     it = __shfl_sync(0xffffffffu, it, 0);
     const int slot = it / nseg, q = it - slot * nseg, s = slot % NS;
-    if (!mbar_wait_or_abort(&full[s], (slot / NS) & 1, wait_limit, vabort)) {
+    if (!__all_sync(0xffffffffu, mbar_wait_or_abort(&full[s], (slot / NS) & 1, wait_limit, vabort))) {
       if (lane == 0 && atomicExch(&abort_flag, 1) == 0) atomicExch(counters + 2, 1ull);
       break;
     }
@@ -599,6 +601,8 @@ k_step_pipe(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
     // slow segment holds its stage only for its loads (the arrival orders them before any
     // later copy into the stage)
     mbar_arrive(&empty[s]);
+    Lanes lanes{};
+    if constexpr (MODE == FIXED) lanes = Lanes{__ballot_sync(0xffffffffu, x < W), G.nx};
     if (x < W) {
       const int n = row * W + x;
       if (G.dirichlet) abb_faces<Elem, R>(g, in, G, x, n, k);
@@ -610,10 +614,10 @@ k_step_pipe(Field<Elem> in, Elem* __restrict__ pout, float* __restrict__ sout, G
       if constexpr (VEL == 2) {
         const R un[3] = {R(__ldg(u3 + n)), R(__ldg(u3 + G.N + n)), R(__ldg(u3 + 2 * G.N + n))};
         tk = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, kc,
-                                             fallback != 0, keep, pr, un);
+                                             fallback != 0, lanes, keep, pr, un);
       } else {
         tk = collide_and_store<R, VEL, MODE>(g, in, pout, sout, G, n, T, T6 != nullptr, r, src, k, kc,
-                                             fallback != 0, keep, pr);
+                                             fallback != 0, lanes, keep, pr);
       }
       took += tk ? 1u : 0u;
       proj += pr ? 1u : 0u;
