@@ -63,8 +63,16 @@ elbm_status elbm2d_set_velocity_uniform(elbm2d_handle h, const double u[2]);
 
 /* Per-node velocity, FP32 [2][N], host or device, copied.  Every node uses the equilibrium
  * and stabilizer tables of its own u (lambda = 1 where that u is exactly 0).  ELBM_ERR_MACH
- * (field discarded) if some node has a P_i(u) <= 0; ELBM_ERR_STATE after initialisation. */
+ * (field discarded) if some node has a P_i(u) <= 0; ELBM_ERR_STATE after initialisation.
+ * An ELBM_F64 handle keeps the tables too, 288 bytes per node, where they take no more than its
+ * table limit and a quarter of the device memory that is free; else every step forms them, with
+ * the same bits. */
 elbm_status elbm2d_set_velocity_field(elbm2d_handle h, const float* u2);
+
+/* Most bytes of tables that this handle keeps (default 8 GiB; 0: none).  Tables that are kept and
+ * larger are freed, also after initialisation; to have them kept again, set the velocity field
+ * again. */
+elbm_status elbm2d_set_table_limit(elbm2d_handle h, size_t bytes);
 
 /* g = g_eq(phi0, u) from phi0 [N] of `dtype`, host or device.  Resets the step counter and
  * the fallback count. */

@@ -364,7 +364,8 @@ __global__ void __launch_bounds__(THREADS2) k_tables2(const float* __restrict__ 
     tab[(size_t)(3 * Q2 + i) * N + n] = k.M[i];
   }
 }
-// Tables larger than this, or than the memory there is, are formed in every step instead.
+// Tables larger than the handle's limit, or than a quarter of the memory that is free, are formed in
+// every step instead.
 constexpr size_t TABLE_BYTES = 8ull << 30;
 
 int elementwise_blocks(size_t N) {
@@ -405,6 +406,7 @@ struct elbm2d_ctx {
   void* T3 = nullptr;          // per-node T field (R), owned
   float* u2 = nullptr;         // per-node velocity [2][N], owned
   double* tab = nullptr;       // its tables (FP64, k_tables2), owned, or null
+  size_t table_limit = TABLE_BYTES;
   bool have_tensor = false, tensor_field = false;
   double D3[3] = {0, 0, 0};
   double u[2] = {0, 0};
@@ -473,6 +475,16 @@ void rebuild(elbm2d_ctx* h) {
 }
 
 size_t esize(int prec) { return prec == 0 ? 8 : 4; }
+
+size_t table_bytes(const elbm2d_ctx* h) { return 4 * Q2 * h->N * sizeof(double); }
+
+// The tables are formed in the steps from now on.
+cudaError_t drop_tables(elbm2d_ctx* h) {
+  const cudaError_t e = cudaStreamSynchronize(h->stream);
+  cudaFree(h->tab);
+  h->tab = nullptr;
+  return e;
+}
 
 // caller array -> device (owned temporary if it was host memory)
 elbm_status to_dev(elbm2d_ctx* h, const void* p, size_t bytes, const void** dev, void** tmp) {
@@ -647,7 +659,15 @@ elbm_status elbm2d_set_tensor_uniform(elbm2d_handle h, const double D3[3]) {
 
 elbm_status elbm2d_set_tensor_field(elbm2d_handle h, const float* D3) {
   if (!h || !D3) return fail(h, ELBM_ERR_ARG, "null argument");
-  if (!h->T3) CK2(cudaMalloc(&h->T3, 3 * h->N * esize(h->prec)), "cudaMalloc T field");
+  if (!h->T3) {
+    cudaError_t e = cudaMalloc(&h->T3, 3 * h->N * esize(h->prec));
+    if (e == cudaErrorMemoryAllocation && h->tab != nullptr) {   // the tables give way
+      cudaGetLastError();
+      CK2(drop_tables(h), "sync");
+      e = cudaMalloc(&h->T3, 3 * h->N * esize(h->prec));
+    }
+    CK2(e, "cudaMalloc T field");
+  }
   const void* dev;
   void* tmp;
   elbm_status s = to_dev(h, D3, 3 * h->N * sizeof(float), &dev, &tmp);
@@ -709,16 +729,27 @@ elbm_status elbm2d_set_velocity_field(elbm2d_handle h, const float* u2) {
   }
   h->u[0] = h->u[1] = 0.0;
   rebuild(h);
-  const size_t bytes = 4 * Q2 * h->N * sizeof(double);
-  if (h->prec == 0 && h->tab == nullptr && bytes <= TABLE_BYTES && cudaMalloc((void**)&h->tab, bytes) != cudaSuccess) {
-    h->tab = nullptr;
-    cudaGetLastError();
+  const size_t bytes = table_bytes(h);
+  if (h->prec == 0 && h->tab == nullptr && bytes <= h->table_limit) {
+    size_t free = 0, total = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess || bytes > free / 4 ||
+        cudaMalloc((void**)&h->tab, bytes) != cudaSuccess) {
+      h->tab = nullptr;
+      cudaGetLastError();
+    }
   }
   if (h->tab != nullptr) {
     k_tables2<<<(unsigned)((h->N + THREADS2 - 1) / THREADS2), THREADS2, 0, h->stream>>>(h->u2, h->tab, h->N);
     CK2(cudaGetLastError(), "velocity tables");
     CK2(cudaStreamSynchronize(h->stream), "sync");   // steps may load them before their wait
   }
+  return ELBM_OK;
+}
+
+elbm_status elbm2d_set_table_limit(elbm2d_handle h, size_t bytes) {
+  if (!h) return ELBM_ERR_ARG;
+  h->table_limit = bytes;
+  if (h->tab != nullptr && table_bytes(h) > bytes) CK2(drop_tables(h), "sync");
   return ELBM_OK;
 }
 

@@ -124,6 +124,7 @@ def lib() -> C.CDLL:
         "elbm2d_set_tensor_field": (S, [H, P]),
         "elbm2d_set_velocity_uniform": (S, [H, D]),
         "elbm2d_set_velocity_field": (S, [H, P]),
+        "elbm2d_set_table_limit": (S, [H, C.c_size_t]),
         "elbm2d_init_equilibrium": (S, [H, P, S]),
         "elbm2d_write_populations": (S, [H, P, S]),
         "elbm2d_read_populations": (S, [H, P, S]),
@@ -574,6 +575,10 @@ def elbm2d_set_velocity_uniform(h, u):
 
 def elbm2d_set_velocity_field(h, u2):
     _check2(lib().elbm2d_set_velocity_field(h, _ptr(u2)), h)
+
+
+def elbm2d_set_table_limit(h, nbytes):
+    _check2(lib().elbm2d_set_table_limit(h, int(nbytes)), h)
 
 
 def elbm2d_init_equilibrium(h, phi0):
