@@ -13,8 +13,9 @@
  * Misfit: J = 1/2 sum_{t in obs} sum_x (phi_t(x) - phi*_t(x))^2 with phi_t the
  * zeroth moment after t steps.  The gradient is computed by a reverse sweep over
  * checkpoints taken every K steps, recomputing each K-step segment forward; runs whose
- * states fit 4 GiB keep them all and recompute nothing.  The handle keeps up to 4 GiB of
- * states between calls.
+ * states fit the handle's workspace (4 GiB unless set otherwise) and half of the device
+ * memory that is free keep them all and recompute nothing.  The handle keeps its states
+ * between calls, up to that size.
  *
  * Arrays are device pointers in the handle's precision (double for ELBM_F64,
  * float for ELBM_F32), layout [component][N] with node n = x + Nx (y + Ny z).
@@ -22,6 +23,7 @@
 #ifndef ELBM_ADJOINT_H
 #define ELBM_ADJOINT_H
 
+#include <stddef.h>
 #include <stdint.h>
 
 #include "elbm.h"
@@ -42,6 +44,11 @@ const char* elbm_adjoint_last_error(elbm_adjoint_handle h);
 /* Velocity (ELBM_ERR_MACH unless all P_i(u) > 0), stabilizer guard theta >= 0,
  * checkpoint interval K >= 1. */
 elbm_status elbm_adjoint_configure(elbm_adjoint_handle h, const double u[3], double theta, int32_t checkpoint_every);
+
+/* Most bytes of states that the handle keeps, within a call instead of checkpoints and
+ * between calls (default 4 GiB).  0: states only at checkpoints every K steps and of one
+ * segment, given back at the end of each call.  What is held above it is freed now. */
+elbm_status elbm_adjoint_set_workspace(elbm_adjoint_handle h, size_t bytes);
 
 /* J (host double) for nsteps steps from g_eq(phi0, u); nobs (1..16) observation
  * steps obs_steps[] in 1..nsteps with targets [nobs][N]; if grad6 != NULL also

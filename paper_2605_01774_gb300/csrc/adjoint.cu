@@ -38,7 +38,8 @@ template <typename R>
 constexpr int STEP_THREADS = sizeof(R) == 8 ? 64 : 128;
 
 // States of a run that are kept rather than recomputed, and the workspace that a handle keeps
-// between calls (a larger one is given back at the end of the call).  64^3 FP32 with 32 steps and
+// between calls (a larger one is given back at the end of the call), unless the caller sets another
+// limit.  64^3 FP32 with 32 steps and
 // checkpoints every 8 (3.1 ms a call) recomputed 28 of them, 14 us each, and got and returned 0.4 GB
 // on each call.
 constexpr size_t KEEP_BYTES = 4ull << 30;
@@ -416,6 +417,7 @@ struct elbm_adjoint_ctx {
   double* aux = nullptr;           // [12][N] (k_params_to_T)
   void* states = nullptr;          // checkpoints and segment states
   size_t state_bytes = 0;
+  size_t keep_bytes = KEEP_BYTES;
   void* gbar[2] = {nullptr, nullptr};
   double* part = nullptr;
   unsigned long long* fb = nullptr;
@@ -513,6 +515,15 @@ cudaError_t vjp(elbm_adjoint_ctx* h, const R* state, const R* gbar_next, R* gbar
                      static_cast<const R*>(h->T6), h->Tbar, target, h->G, kc<R>(h), first ? 1 : 0);
 }
 
+// Whether all states of a run may be kept: within the handle's limit, and within half of the memory
+// that is free for them.
+bool may_keep(const elbm_adjoint_ctx* h, size_t bytes) {
+  if (bytes > h->keep_bytes) return false;
+  if (bytes <= h->state_bytes) return true;
+  size_t free = 0, total = 0;
+  return cudaMemGetInfo(&free, &total) == cudaSuccess && bytes <= (free + h->state_bytes) / 2;
+}
+
 // Room for `bytes` of states in the handle's workspace.
 cudaError_t reserve(elbm_adjoint_ctx* h, size_t bytes) {
   if (bytes <= h->state_bytes) return cudaSuccess;
@@ -533,8 +544,8 @@ elbm_status run_steps(elbm_adjoint_ctx* h, const R* theta, const R* phi0, int64_
   const size_t S = 27ull * N, sb = S * sizeof(R);
   cudaStream_t s = h->stream;
   // Segments of K steps.  A forward run alone alternates between two states.  With a gradient, every
-  // state of the run is kept if they fit KEEP_BYTES (one segment); else checkpoints every
-  // h->K steps, and the states of one segment at a time.
+  // state of the run is kept where that is allowed (one segment); else checkpoints every h->K steps,
+  // and the states of one segment at a time.
   int64_t K = nsteps, last = 0, t_last = 0;     // last segment, its first step
   size_t ncheck = 1, nseg = 2;
   const auto plan = [&](int64_t every) {
@@ -544,7 +555,8 @@ elbm_status run_steps(elbm_adjoint_ctx* h, const R* theta, const R* phi0, int64_
     ncheck = (size_t)last + 1;
     nseg = (size_t)K + 1;
   };
-  if (grad != nullptr) plan((size_t)(nsteps + 2) <= KEEP_BYTES / sb ? nsteps : h->K);
+  if (grad != nullptr)
+    plan(nsteps > h->K && (size_t)(nsteps + 2) <= h->keep_bytes / sb && may_keep(h, (size_t)(nsteps + 2) * sb) ? nsteps : h->K);
   cudaError_t e = reserve(h, (ncheck + nseg) * sb);
   if (e == cudaErrorMemoryAllocation && grad != nullptr && K > h->K) {
     plan(h->K);
@@ -614,16 +626,18 @@ elbm_status run_steps(elbm_adjoint_ctx* h, const R* theta, const R* phi0, int64_
   return ELBM_OK;
 }
 
+void release_states(elbm_adjoint_ctx* h) {
+  cudaStreamSynchronize(h->stream);
+  cudaFree(h->states);
+  h->states = nullptr;
+  h->state_bytes = 0;
+}
+
 template <typename R>
 elbm_status run_t(elbm_adjoint_ctx* h, const R* theta, const R* phi0, int64_t nsteps, int nobs, const int64_t* obs,
                   const R* targets, double* J, R* grad, int64_t* nfb) {
   const elbm_status st = run_steps<R>(h, theta, phi0, nsteps, nobs, obs, targets, J, grad, nfb);
-  if (h->state_bytes > KEEP_BYTES) {
-    cudaStreamSynchronize(h->stream);
-    cudaFree(h->states);
-    h->states = nullptr;
-    h->state_bytes = 0;
-  }
+  if (h->state_bytes > h->keep_bytes) release_states(h);
   return st;
 }
 
@@ -683,6 +697,13 @@ elbm_status elbm_adjoint_configure(elbm_adjoint_handle h, const double u[3], dou
   h->theta = theta;
   h->K = checkpoint_every;
   consts_for(h);
+  return ELBM_OK;
+}
+
+elbm_status elbm_adjoint_set_workspace(elbm_adjoint_handle h, size_t bytes) {
+  if (!h) return ELBM_ERR_ARG;
+  h->keep_bytes = bytes;
+  if (h->state_bytes > bytes) release_states(h);
   return ELBM_OK;
 }
 

@@ -112,6 +112,7 @@ def lib() -> C.CDLL:
         "elbm_adjoint_destroy": (None, [H]),
         "elbm_adjoint_last_error": (C.c_char_p, [H]),
         "elbm_adjoint_configure": (S, [H, D, C.c_double, I32]),
+        "elbm_adjoint_set_workspace": (S, [H, C.c_size_t]),
         "elbm_adjoint_misfit": (S, [H, P, P, I64, I32, PI64, P, D, P, PI64]),
         "elbm_adjoint_step": (S, [H, P, P, P, P, P, P]),
     })
@@ -451,6 +452,10 @@ def elbm_adjoint_destroy(h):
 
 def elbm_adjoint_configure(h, u, theta=1e-8, checkpoint_every=50):
     _acheck(lib().elbm_adjoint_configure(h, _d(u, 3), float(theta), int(checkpoint_every)), h)
+
+
+def elbm_adjoint_set_workspace(h, nbytes):
+    _acheck(lib().elbm_adjoint_set_workspace(h, int(nbytes)), h)
 
 
 def elbm_adjoint_misfit(h, theta6, phi0, nsteps, obs_steps, targets, grad6=None):
