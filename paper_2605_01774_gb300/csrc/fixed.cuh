@@ -5,9 +5,11 @@
 // the time of an FP64 step (17 times its DRAM time).  In fixed point relative to the node's
 // largest population the sums are exact, the products are four 32-bit multiplications,
 // and only the quotient kappa takes (FP32) floating point, refined by integer remainders.
-// Measured per step: 128^3 plume 2.1 -> 0.72 ms, 96 x 80 x 72 plume 0.511 -> 0.16 ms, 128^3 with
-// tensor field and source 1.80 -> 0.59 ms.  What bounds it now is instruction issue (6800 per warp,
-// 56 % of the slots) with 12 warps per SM, at 0.18 of the DRAM rate.
+// Measured per step: 96 x 80 x 72 plume 0.511 -> 0.16 ms, 128^3 with tensor field and source 1.80 ->
+// 0.59 ms, the first steps of a 128^3 plume 2.1 -> 0.72 ms.  What bounds it now is instruction issue
+// (6800 per warp, 56 % of the slots) with 12 warps per SM, at 0.18 of the DRAM rate.  Steep tails are
+// left to FP64 (collide64.cuh), where they make up most of a box at little gain: the 256^3 plume 8
+// nodes wide takes 13.1 to 17.7 ms a step where FP64 arithmetic takes 17.8 to 20.1.
 //
 // Representation: population i is held as 4^n_i g_i, n_i its number of nonzero velocity components
 // (all of them about 8/27 phi near equilibrium, W_i = 8/27 4^-n_i), in units U = 2^(etop - 57),
@@ -17,7 +19,8 @@
 //     8/9 |c.(a - j)| <= 14 t < 2^62.
 // U is 1e-18 to 3e-18 of phi near equilibrium, a tenth of the FP64 rounding of the rest population,
 // so the result (rounded to FP64 once, at the end) is closer to the exact collision than FP64
-// arithmetic gives.
+// arithmetic gives.  Populations below t/32 lose the bits under the unit; where that would tell in the
+// others, in the fallback's alpha, they are read again (blend_given).
 //
 // With 3 W_i = (8/9) 4^-n_i, and m = sum c g = j + phi u,
 //     4^n b_i  = 4^n (phi E_i + 3 W_i c.j) = 8/27 phi (1 - 1.5 u.u + 4.5 (c.u)^2) + c.(8/9 m),
@@ -455,13 +458,10 @@ ELBM_HD Fixed collide_fixed(const double (&v)[Q], const double* Tn, double src, 
   {
     if (Tn != nullptr) {
       // T = 2I - S < 2, but rounds to 2 and a little above for D of 5e14 and more
-      uint32_t most = 0;
+      uint32_t any = 0;
 #pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        const uint32_t h = (uint32_t)(bits_of(Tn[q]) >> 32) & 0x7fffffffu;
-        most = h > most ? h : most;
-      }
-      if (most >= 0x40000000u) return Fixed::REFUSED;   // some |T| >= 2, or NaN
+      for (int q = 0; q < 6; ++q) any |= (uint32_t)(bits_of(Tn[q]) >> 32);
+      if ((any & 0x40000000u) != 0) return Fixed::REFUSED;   // the exponent of some |T| >= 2, or NaN
     }
     Q64 T[6];
 #pragma unroll
